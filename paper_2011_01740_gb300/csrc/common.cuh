@@ -167,6 +167,9 @@ enum Pair : int { kCashKarp = 0, kDormandPrince = 1 };
 // their step counts, so it runs at max(tol, 1e-7): a quarter of the steps of a
 // 1e-10 pilot, and the claim order never changes what a system computes.
 constexpr double kPilotTol = 1e-7;
+// Most trials of one system in a split-precision pilot (a forcing period takes
+// the hardest systems of the p_A x f maps about 1,000 at kPilotTol).
+constexpr int64_t kPilotTrials = 1 << 14;
 
 // Host helpers of abi.cu shared with the other entry points.
 // Validates the solver settings of an adaptive or fixed-step solve; on failure
