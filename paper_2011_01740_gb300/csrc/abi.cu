@@ -92,24 +92,57 @@ ens_status cuda_fail(ens_ctx* c, cudaError_t e, const char* what) {
     if (e_ != cudaSuccess) return cuda_fail((ctx), e_, #call);       \
   } while (0)
 
+// The launch of a context whose caller sets none.  Every line lies between
+// measured shapes (GB300, 152 SMs; milliseconds of a whole pass, horizons of 2
+// to 6 periods or 16 time units); all shapes give the same results.
+//   Up to one warp per SM sub-partition (128 systems per SM) every system
+//   starts at once, so an order only costs its pilot, and blocks of one warp
+//   put each warp on a sub-partition of its own: 1,073 bubbles 45.4 against
+//   51.7 (160 x 1, longest first), 15,000 45.6 / 52.7, 4,608 frequencies 141.7 /
+//   147.7, split precision 16,384 14.4 / 17.4.
+//   Above that the longest systems bound the run until there are enough
+//   others; FP64 phases want 5 warps per SM (65,536 systems: 57.6, 6 warps
+//   58.9), then 6 (131,044: 207 / 221 at 5), then 12 (262,144: 122 / 149;
+//   524,288: 236 / 295).  Split precision: 8 (131,044: 19.1 / 20.4), 12
+//   (262,144: 23.6 / 38.2), 16 (524,288: 37.9 / 74.9), 24 from there.
+//   Double-float phases 4 (65,536: 93.6 / 94.9), then 8 (131,044: 110 / 133;
+//   262,144: 105 / 145).
+//   Valves take about the same number of steps each, and neighbours take them
+//   alike, which claiming by cost breaks up: plain launches of 1 warp a block
+//   (1,000: 21.6 / 25.4; 32,768: 26.4 / 37.2; 65,536: 47.8 / 60.7), of 2 for the
+//   larger ensembles (262,144: 173 / 211); double-float ones, whose unrolled
+//   trial is bound by instruction fetch, of 8 (131,072: 39.7 / 94.0; 524,288:
+//   138 / 352).
 ens_launch default_launch(const ens_ctx* c) {
   ens_launch L{};
-  if (c->solver == ENS_RK4) {
-    L.mode = ENS_LAUNCH_PLAIN;
-    L.block = 32;
-    L.blocks_per_sm = 0;
-  } else {
-    // about one warp per SM sub-partition saturates the FP64 pipe.  More warps
-    // share the pipe and lengthen the critical path of the longest system
-    // (each warp then advances more slowly); fewer leave the pipe idle on
-    // dependent-instruction latency.  Five warps per SM measured fastest on
-    // the 362 x 362 Keller-Miksis sweep, with longest-first claiming.
-    L.mode = ENS_LAUNCH_PERSISTENT;
-    L.block = 160;
-    L.blocks_per_sm = 1;
-    L.cost_order = 1;
+  L.mode = ENS_LAUNCH_PLAIN;
+  L.block = 32;
+  const int64_t per_sm = c->n / std::max(1, c->sm_count);  // systems per SM
+  if (c->solver == ENS_RK4) return L;
+  if (c->sys == ENS_SYS_RELIEF_VALVE && c->tol.n_phases == 0) {
+    if (c->tol.prec == ENS_FP32X2) L.block = 256;
+    else if (per_sm >= 512) L.block = 64;
+    return L;
   }
-  L.use_graph = 0;
+  if (c->n <= (int64_t)c->sm_count * 128) {
+    // the double-float trial is bound by instruction fetch, which warps of one SM share
+    if (c->tol.prec == ENS_FP32X2) L.block = 128;
+    return L;
+  }
+  L.mode = ENS_LAUNCH_PERSISTENT;
+  L.blocks_per_sm = 1;
+  L.cost_order = 1;
+  if (c->tol.prec == ENS_FP32_COMP) {
+    L.block = per_sm >= 1300 && per_sm < 2600 ? 128 : 256;
+    L.blocks_per_sm = per_sm < 1300 ? 1 : per_sm < 2600 ? 3 : per_sm < 5200 ? 2 : 3;
+  } else if (c->tol.prec == ENS_FP32X2) {
+    L.block = per_sm < 640 ? 128 : 256;
+  } else if (per_sm < 1300) {
+    L.block = per_sm < 640 ? 160 : 192;
+  } else {
+    L.block = 128;
+    L.blocks_per_sm = 3;
+  }
   return L;
 }
 

@@ -66,7 +66,8 @@ def km_solve_labels(ens, phys: dict, liquid: dict, n_phases: int, first_phase: i
                         timeout_s=1800.0)
     ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS, n, C, y0, (0.0, 1.0), ens.ENS_RKCK45, ttol)
     try:
-        ens.ens_set_launch(ctx, launch or ens.make_launch(block=160, blocks_per_sm=1, cost_order=1))
+        if launch is not None:
+            ens.ens_set_launch(ctx, launch)
         ens.ens_solve(ctx, stream)
         st = ens.ens_sync(ctx)
         acc = torch.empty((2 * n_phases, n), dtype=torch.float64, device=dev)
