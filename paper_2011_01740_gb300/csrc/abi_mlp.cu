@@ -23,21 +23,22 @@ struct ens_mlp {
   float* m2 = nullptr;
   float* grad = nullptr;
   int64_t adam_t = 0;
-  // batch scratch
+  // batch scratch for the products it was made for (train_impl at the time)
   int64_t cap = 0;
+  int cap_impl = -1;
   float* xb = nullptr;
   float* yb = nullptr;
-  float* z = nullptr;
-  float* gp = nullptr;            // gelu'(z) of the tcgen05 forward, [members][B][4][128]
+  float* z = nullptr;             // mma.sync: [members][B][4][128] pre-activations
   float* dz = nullptr;
   float* out = nullptr;
   float* dout = nullptr;
-  float* loss = nullptr;          // [members]
+  // [members] loss sums, then the error word of the tcgen05 kernels: read back together
+  float* loss = nullptr;
   float* gpart = nullptr;         // [kMaxSplits][members][kP] partial gradients of the batch slices
+  float* block = nullptr;         // tcgen05: FP32 dz and gelu(z_4), see TrainTcArgs
+  __nv_bfloat16* tile = nullptr;  // tcgen05: operand tiles, see TrainTcArgs
   // training products: 1 tcgen05 kernels (mlp_tc05_train.cu), 0 mma.sync kernels (mlp.cu)
   int train_impl = 1;
-  unsigned* train_err = nullptr;  // set by a tcgen05 training kernel whose wait expired
-  __nv_bfloat16* wbfT = nullptr;  // [members][3][128][128] transposed hidden weights (tcgen05 backward)
   // screening on the tcgen05 tensor cores
   int screen_impl = 1;            // 1: tcgen05 kernel, 0: mma.sync fused kernel
   float* screen_out = nullptr;    // [members][screen_cap][2]
@@ -76,131 +77,146 @@ bool is_device(const void* p) {
   return ok && (at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged);
 }
 
+// memory that a kernel on the current device may address directly (device
+// memory of another GPU would be a peer address)
+bool is_local(const void* p) {
+  cudaPointerAttributes at{};
+  int dev = -1;
+  const bool ok = cudaPointerGetAttributes(&at, p) == cudaSuccess && cudaGetDevice(&dev) == cudaSuccess;
+  cudaGetLastError();
+  return ok && (at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == dev));
+}
+
 unsigned grid_for(int64_t n, int block = 256, int64_t cap = 8192) {
   int64_t g = (n + block - 1) / block;
   if (g < 1) g = 1;
   return (unsigned)std::min<int64_t>(g, cap);
 }
 
-ens_status ensure_batch(ens_mlp* m, int64_t B) {
-  if (B <= m->cap) return ENS_OK;
+unsigned* train_err(const ens_mlp* m) { return reinterpret_cast<unsigned*>(m->loss + m->members); }
+
+void free_batch(ens_mlp* m) {
   cudaFree(m->xb);
   cudaFree(m->yb);
   cudaFree(m->z);
-  cudaFree(m->gp);
   cudaFree(m->dz);
+  cudaFree(m->block);
+  cudaFree(m->tile);
   cudaFree(m->out);
   cudaFree(m->dout);
-  m->xb = m->yb = m->z = m->gp = m->dz = m->out = m->dout = nullptr;
+  m->xb = m->yb = m->z = m->dz = m->block = m->out = m->dout = nullptr;
+  m->tile = nullptr;
   m->cap = 0;
+}
+
+// most operand tiles of a batch of up to B samples: each of the slices may end
+// in a ragged tile
+int64_t most_tiles(int64_t B) { return (B + mlp::kTile - 1) / mlp::kTile + 2 * mlp::kMaxSplits; }
+
+// scratch of a batch of up to B samples for the selected products
+ens_status ensure_batch(ens_mlp* m, int64_t B) {
+  if (B <= m->cap && m->cap_impl == m->train_impl) return ENS_OK;
+  free_batch(m);
   const size_t M = (size_t)m->members;
-  cudaError_t e = cudaMalloc(&m->xb, B * 2 * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&m->yb, B * 2 * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&m->z, M * B * 4 * mlp::H * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&m->gp, M * B * 4 * mlp::H * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&m->dz, M * 4 * B * mlp::H * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&m->out, M * B * 2 * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&m->dout, M * B * 2 * sizeof(float));
+  const bool tc = m->train_impl == 1;
+  const size_t pairs = (size_t)mlp::pair_rows(B) * 2 * sizeof(float);
+  cudaError_t e = cudaMalloc(&m->xb, pairs);
+  if (e == cudaSuccess) e = cudaMalloc(&m->yb, pairs);
+  if (e == cudaSuccess) e = cudaMalloc(&m->dout, M * pairs);
+  if (e == cudaSuccess && tc) e = cudaMalloc(&m->block, M * most_tiles(B) * 5 * 4 * mlp::kBlock * sizeof(float));
+  if (e == cudaSuccess && tc)
+    e = cudaMalloc(&m->tile, M * most_tiles(B) * 6 * mlp::H * mlp::H * sizeof(__nv_bfloat16));
+  if (e == cudaSuccess && !tc) e = cudaMalloc(&m->dz, M * 4 * B * mlp::H * sizeof(float));
+  if (e == cudaSuccess && !tc) e = cudaMalloc(&m->z, M * B * 4 * mlp::H * sizeof(float));
+  if (e == cudaSuccess && !tc) e = cudaMalloc(&m->out, M * B * 2 * sizeof(float));
   if (e == cudaSuccess && !m->gpart)
     e = cudaMalloc(&m->gpart, (size_t)mlp::kMaxSplits * M * mlp::kP * sizeof(float));
-  if (e == cudaSuccess && !m->wbfT) e = cudaMalloc(&m->wbfT, M * 3 * mlp::H * mlp::H * sizeof(__nv_bfloat16));
-  if (e == cudaSuccess && !m->train_err) {
-    e = cudaMalloc(&m->train_err, sizeof(unsigned));
-    if (e == cudaSuccess) e = cudaMemset(m->train_err, 0, sizeof(unsigned));
-  }
   if (e != cudaSuccess) {
     merr(m, "batch scratch: %s", cudaGetErrorString(e));
     return ENS_ENOMEM;
   }
   m->cap = B;
+  m->cap_impl = m->train_impl;
   return ENS_OK;
 }
 
-// arguments of the tcgen05 training kernels over the batch scratch
-mlp::TrainTcArgs tc_args(ens_mlp* m, int64_t B, const float* x, float* out, float* loss, int64_t rows) {
-  mlp::TrainTcArgs t{};
-  t.n = B;
-  t.members = m->members;
-  t.x = x;
-  t.y = m->yb;
-  t.master = m->master;
-  t.wbf = m->wbf;
-  t.wbfT = m->wbfT;
-  t.z = m->z;
-  t.gp = m->gp;
-  t.out = out;
-  t.dout = m->dout;
-  t.dz = m->dz;
-  t.loss = loss;
-  t.grad = m->gpart;
-  t.rows = rows;
-  t.error = m->train_err;
-  return t;
-}
-
-// forward (training form) + backward + weight gradients of one batch already
-// in m->xb / m->yb; loss[members] accumulates the per-sample loss sum.  The
-// gradient is left as slice partials in m->gpart, their number in *splits;
-// with splits == nullptr they are summed into m->grad.
-ens_status batch_grad(ens_mlp* m, int64_t B, float* loss, cudaStream_t s, int* splits_out) {
-  const int splits = mlp::grad_splits(B);
-  const int64_t rows = ((B + splits - 1) / splits + mlp::kChunk - 1) / mlp::kChunk * mlp::kChunk;
+// Loss and gradient of one batch, rows perm[0..B) of x and y (0..B-1 for a null
+// perm); loss[members] accumulates the per-sample loss sum.  The gradient is
+// left as partials in m->gpart, their number in *splits.
+ens_status batch_grad(ens_mlp* m, int64_t B, const float* x, const float* y, const int32_t* perm, float* loss,
+                      cudaStream_t s, int* splits) {
+  *splits = mlp::grad_splits(B);
+  const int64_t rows = mlp::slice_rows(B, *splits);
   if (m->train_impl == 1) {
-    // tcgen05: forward, input gradients, weight gradients (the 2-wide layers
-    // 1 and 5 in FP32 by blocks of the same launch)
-    const mlp::TrainTcArgs t = tc_args(m, B, m->xb, m->out, loss, rows);
-    MLP_CUDA(m, mlp::launch_train_tc05(0, t, splits, s));
-    MLP_CUDA(m, mlp::launch_train_tc05(1, t, splits, s));
-    MLP_CUDA(m, mlp::launch_train_tc05(2, t, splits, s));
-  } else {
-    mlp::FwdArgs f{};
-    f.n = B;
-    f.members = m->members;
-    f.x = m->xb;
-    f.master = m->master;
-    f.wbf = m->wbf;
-    f.z = m->z;
-    f.out = m->out;
-    MLP_CUDA(m, mlp::launch_forward_train(f, s));
-    mlp::BwdArgs b{};
-    b.n = B;
-    b.y = m->yb;
-    b.master = m->master;
-    b.wbf = m->wbf;
-    b.z = m->z;
-    b.out = m->out;
-    b.dout = m->dout;
-    b.dz = m->dz;
-    b.loss = loss;
-    MLP_CUDA(m, mlp::launch_backward(b, m->members, s));
-    mlp::GradArgs g{};
-    g.n = B;
-    g.x = m->xb;
-    g.z = m->z;
-    g.dz = m->dz;
-    g.dout = m->dout;
-    g.grad = m->gpart;
-    g.rows = rows;
-    MLP_CUDA(m, mlp::launch_wgrad(g, m->members, splits, s));
+    mlp::TrainTcArgs t{};
+    t.n = B;
+    t.members = m->members;
+    t.x = x;
+    t.y = y;
+    t.perm = perm;
+    t.master = m->master;
+    t.wbf = m->wbf;
+    t.rows = rows;
+    t.tiles = mlp::step_tiles(rows, *splits);
+    t.tile = m->tile;
+    t.block = m->block;
+    t.dout = m->dout;
+    t.xb = m->xb;
+    t.loss = loss;
+    t.grad = m->gpart;
+    t.error = train_err(m);
+    MLP_CUDA(m, mlp::launch_step_tc05(t, *splits, m->sms, s));
+    return ENS_OK;
   }
-  if (splits_out)
-    *splits_out = splits;
-  else
-    MLP_CUDA(m, mlp::launch_grad_reduce(m->members, splits, m->gpart, m->grad, s));
+  if (perm) {
+    MLP_CUDA(m, mlp::launch_gather(B, perm, x, y, m->xb, m->yb, s));
+    x = m->xb;
+    y = m->yb;
+  }
+  mlp::FwdArgs f{};
+  f.n = B;
+  f.members = m->members;
+  f.x = x;
+  f.master = m->master;
+  f.wbf = m->wbf;
+  f.z = m->z;
+  f.out = m->out;
+  MLP_CUDA(m, mlp::launch_forward_train(f, s));
+  mlp::BwdArgs b{};
+  b.n = B;
+  b.y = y;
+  b.master = m->master;
+  b.wbf = m->wbf;
+  b.z = m->z;
+  b.out = m->out;
+  b.dout = m->dout;
+  b.dz = m->dz;
+  b.loss = loss;
+  MLP_CUDA(m, mlp::launch_backward(b, m->members, s));
+  mlp::GradArgs g{};
+  g.n = B;
+  g.x = x;
+  g.z = m->z;
+  g.dz = m->dz;
+  g.dout = m->dout;
+  g.grad = m->gpart;
+  g.rows = rows;
+  MLP_CUDA(m, mlp::launch_wgrad(g, m->members, *splits, s));
   return ENS_OK;
+}
+
+ens_status expired(ens_mlp* m) {
+  merr(m, "tcgen05 training kernel: wait for the tensor cores expired");
+  return ENS_ECUDA;
 }
 
 // after a synchronous call: a tcgen05 training kernel that gave up waiting
 // for its tensor cores leaves invalid results
 ens_status check_train_err(ens_mlp* m) {
-  if (m->train_impl != 1 || !m->train_err) return ENS_OK;
+  if (m->train_impl != 1) return ENS_OK;
   unsigned e = 0;
-  MLP_CUDA(m, cudaMemcpy(&e, m->train_err, sizeof(unsigned), cudaMemcpyDeviceToHost));
-  if (e) {
-    merr(m, "tcgen05 training kernel: wait for the tensor cores expired");
-    return ENS_ECUDA;
-  }
-  return ENS_OK;
+  MLP_CUDA(m, cudaMemcpy(&e, train_err(m), sizeof(unsigned), cudaMemcpyDeviceToHost));
+  return e ? expired(m) : ENS_OK;
 }
 
 ens_status set_smem_attrs(ens_mlp* m) {
@@ -380,7 +396,11 @@ ens_status ens_mlp_create(ens_mlp** out, int32_t members, uint64_t seed) {
   if (e == cudaSuccess) e = cudaMalloc(&m->m1, tot * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&m->m2, tot * sizeof(float));
   if (e == cudaSuccess) e = cudaMalloc(&m->grad, tot * sizeof(float));
-  if (e == cudaSuccess) e = cudaMalloc(&m->loss, (size_t)members * sizeof(float));
+  if (e == cudaSuccess) e = cudaMalloc(&m->loss, (size_t)(members + 1) * sizeof(float));
+  if (e == cudaSuccess) e = cudaMemset(m->loss, 0, (size_t)(members + 1) * sizeof(float));
+  int dev = 0;
+  if (e == cudaSuccess) e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev);
   if (e == cudaSuccess) e = cudaMemset(m->m1, 0, tot * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(m->m2, 0, tot * sizeof(float));
   if (e == cudaSuccess) e = cudaMemset(m->grad, 0, tot * sizeof(float));
@@ -443,12 +463,12 @@ ens_status ens_mlp_forward(ens_mlp* m, int64_t n, const float* x, float* out, vo
     return ENS_EINVAL;
   }
   cudaStream_t s = (cudaStream_t)stream;
-  ens_status st = ensure_batch(m, n);
-  if (st != ENS_OK) return st;
   if (m->train_impl == 1) {
-    MLP_CUDA(m, mlp::launch_train_tc05(0, tc_args(m, n, x, out, m->loss, n), 1, s));
+    MLP_CUDA(m, mlp::launch_forward_tc05(n, m->members, x, m->master, m->wbf, out, train_err(m), m->sms, s));
     return ENS_OK;
   }
+  ens_status st = ensure_batch(m, n);
+  if (st != ENS_OK) return st;
   mlp::FwdArgs f{};
   f.n = n;
   f.members = m->members;
@@ -471,18 +491,27 @@ ens_status ens_mlp_loss_grad(ens_mlp* m, int64_t n, const float* x, const float*
   cudaStream_t s = (cudaStream_t)stream;
   ens_status st = ensure_batch(m, n);
   if (st != ENS_OK) return st;
-  MLP_CUDA(m, cudaMemcpyAsync(m->xb, x, n * 2 * sizeof(float), cudaMemcpyDeviceToDevice, s));
-  MLP_CUDA(m, cudaMemcpyAsync(m->yb, y, n * 2 * sizeof(float), cudaMemcpyDeviceToDevice, s));
-  MLP_CUDA(m, cudaMemsetAsync(m->loss, 0, m->members * sizeof(float), s));
-  MLP_CUDA(m, cudaMemsetAsync(m->train_err, 0, sizeof(unsigned), s));
-  st = batch_grad(m, n, m->loss, s, nullptr);
+  MLP_CUDA(m, cudaMemsetAsync(m->loss, 0, (m->members + 1) * sizeof(float), s));
+  if (!is_local(x) || !is_local(y)) {   // samples in another GPU's memory are copied over first
+    MLP_CUDA(m, cudaMemcpyAsync(m->xb, x, n * 2 * sizeof(float), cudaMemcpyDefault, s));
+    MLP_CUDA(m, cudaMemcpyAsync(m->yb, y, n * 2 * sizeof(float), cudaMemcpyDefault, s));
+    x = m->xb;
+    y = m->yb;
+  }
+  int splits = 1;
+  st = batch_grad(m, n, x, y, nullptr, m->loss, s, &splits);
   if (st != ENS_OK) return st;
-  std::vector<float> l(m->members);
-  MLP_CUDA(m, cudaMemcpyAsync(l.data(), m->loss, m->members * sizeof(float), cudaMemcpyDeviceToHost, s));
-  MLP_CUDA(m, cudaMemcpyAsync(grad, m->grad, (size_t)m->members * mlp::kP * sizeof(float), cudaMemcpyDefault, s));
+  // straight into the caller's array where a kernel can write it, else through m->grad
+  const bool direct = is_local(grad);
+  MLP_CUDA(m, mlp::launch_grad_reduce(m->members, splits, m->gpart, direct ? grad : m->grad, s));
+  float l[mlp::kMaxMembers + 1];
+  MLP_CUDA(m, cudaMemcpyAsync(l, m->loss, (m->members + 1) * sizeof(float), cudaMemcpyDeviceToHost, s));
+  if (!direct)
+    MLP_CUDA(m, cudaMemcpyAsync(grad, m->grad, (size_t)m->members * mlp::kP * sizeof(float), cudaMemcpyDefault, s));
   MLP_CUDA(m, cudaStreamSynchronize(s));
-  st = check_train_err(m);
-  if (st != ENS_OK) return st;
+  unsigned err = 0;
+  memcpy(&err, l + m->members, sizeof(unsigned));
+  if (m->train_impl == 1 && err) return expired(m);
   for (int k = 0; k < m->members; ++k) loss[k] = l[k] / (float)n;
   return ENS_OK;
 }
@@ -510,9 +539,8 @@ ens_status ens_mlp_train(ens_mlp* m, int64_t n, const float* x, const float* y, 
     return ENS_ENOMEM;
   }
   e = cudaMemsetAsync(hist_d, 0, (size_t)std::max(1, cfg->epochs) * m->members * sizeof(float), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(m->train_err, 0, sizeof(unsigned), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(train_err(m), 0, sizeof(unsigned), s);
   std::vector<int32_t> perm(n);
-  const int64_t tot = (int64_t)m->members * mlp::kP;
   const int64_t steps_total = (int64_t)cfg->epochs * ((n + B - 1) / B);
   int64_t step = 0;
   for (int ep = 0; ep < cfg->epochs && e == cudaSuccess; ++ep) {
@@ -527,10 +555,8 @@ ens_status ens_mlp_train(ens_mlp* m, int64_t n, const float* x, const float* y, 
     e = cudaMemcpyAsync(perm_d, perm.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, s);
     for (int64_t b0 = 0; b0 < n && e == cudaSuccess; b0 += B) {
       const int64_t nb = std::min<int64_t>(B, n - b0);
-      e = mlp::launch_gather(nb, perm_d + b0, x, y, m->xb, m->yb, s);
-      if (e != cudaSuccess) break;
       int splits = 1;
-      st = batch_grad(m, nb, hist_d + (size_t)ep * m->members, s, &splits);
+      st = batch_grad(m, nb, x, y, perm_d + b0, hist_d + (size_t)ep * m->members, s, &splits);
       if (st != ENS_OK) break;
       m->adam_t += 1;
       const float c1 = 1.0f - powf(cfg->beta1, (float)m->adam_t);
@@ -542,7 +568,7 @@ ens_status ens_mlp_train(ens_mlp* m, int64_t n, const float* x, const float* y, 
         lr = (float)(cfg->lr_final + 0.5 * (cfg->lr - cfg->lr_final) * (1.0 + cos(3.14159265358979323846 * x)));
       }
       ++step;
-      e = mlp::launch_adam(tot, m->master, m->wbf, m->gpart, splits, m->m1, m->m2, lr, cfg->beta1, cfg->beta2,
+      e = mlp::launch_adam(m->members, m->master, m->wbf, m->gpart, splits, m->m1, m->m2, lr, cfg->beta1, cfg->beta2,
                            cfg->eps, c1, c2, s);
     }
     if (st != ENS_OK) break;
@@ -585,11 +611,6 @@ ens_status ens_mlp_screen(ens_mlp* m, int64_t n, const float* x, float* mean, fl
       m->screen_cap = n;
     }
     if (!m->screen_err) MLP_CUDA(m, cudaMalloc(&m->screen_err, sizeof(unsigned)));
-    if (!m->sms) {
-      int dev = 0;
-      MLP_CUDA(m, cudaGetDevice(&dev));
-      MLP_CUDA(m, cudaDeviceGetAttribute(&m->sms, cudaDevAttrMultiProcessorCount, dev));
-    }
     MLP_CUDA(m, cudaMemsetAsync(m->screen_err, 0, sizeof(unsigned), s));
     MLP_CUDA(m, mlp::launch_screen_tc05(n, m->members, x, m->master, m->wbf, m->screen_out, m->screen_err, mean,
                                         stdv, p1, m->sms, s));
@@ -623,7 +644,7 @@ ens_status ens_mlp_set_train_impl(ens_mlp* m, int32_t impl, int32_t* wait_expire
   if (!m || (impl != 0 && impl != 1)) return ENS_EINVAL;
   if (wait_expired) {
     unsigned e = 0;
-    if (m->train_err) MLP_CUDA(m, cudaMemcpy(&e, m->train_err, sizeof(unsigned), cudaMemcpyDeviceToHost));
+    MLP_CUDA(m, cudaMemcpy(&e, train_err(m), sizeof(unsigned), cudaMemcpyDeviceToHost));
     *wait_expired = (int32_t)e;
   }
   m->train_impl = impl;
@@ -641,17 +662,9 @@ void ens_mlp_destroy(ens_mlp* m) {
   cudaFree(m->grad);
   cudaFree(m->loss);
   cudaFree(m->gpart);
-  cudaFree(m->xb);
-  cudaFree(m->yb);
-  cudaFree(m->z);
-  cudaFree(m->gp);
-  cudaFree(m->dz);
-  cudaFree(m->out);
-  cudaFree(m->dout);
+  free_batch(m);
   cudaFree(m->screen_out);
   cudaFree(m->screen_err);
-  cudaFree(m->train_err);
-  cudaFree(m->wbfT);
   delete m;
 }
 

@@ -320,22 +320,46 @@ __global__ void __launch_bounds__(kThreads) mlp_wgrad_kernel(GradArgs a) {
 }
 
 
-// Adam (Kingma & Ba 2015) on the FP32 master weights; refreshes the BF16 copy.
-// Adam step; the gradient is the sum of the slice partials part[k][i], k in
-// order (the same sums as mlp_grad_reduce_kernel)
-__global__ void adam_kernel(int64_t total, float* w, __nv_bfloat16* wb, const float* part, int splits, float* m1,
-                            float* m2, float lr, float b1, float b2, float eps, float c1, float c2) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    float gi = part[i];
-    for (int k = 1; k < splits; ++k) gi += part[(int64_t)k * total + i];
-    const float a = fmaf(b1, m1[i], (1.0f - b1) * gi);
-    const float v = fmaf(b2, m2[i], (1.0f - b2) * gi * gi);
-    m1[i] = a;
-    m2[i] = v;
-    const float upd = lr * (a / c1) / (sqrtf(v / c2) + eps);
-    w[i] -= upd;
-    wb[(i / kP) * kPS + i % kP] = __float2bfloat16(w[i]);
+// Sum over the partials part[k][total] of the parameter pair at element i, k
+// in order; the loads of eight partials are in flight together.
+__device__ __forceinline__ float2 partial_sum(const float* part, int64_t total, int splits, int64_t i) {
+  float2 g = *reinterpret_cast<const float2*>(part + i);
+#pragma unroll 8
+  for (int k = 1; k < splits; ++k) {
+    const float2 q = *reinterpret_cast<const float2*>(part + (int64_t)k * total + i);
+    g.x += q.x;
+    g.y += q.y;
   }
+  return g;
+}
+
+// Adam (Kingma & Ba 2015) on the FP32 master weights; refreshes the BF16
+// copy.  grid.y = member, thread = two neighbouring parameters.
+__device__ __forceinline__ float adam_one(float w, float gi, float& m1, float& m2, float lr, float b1, float b2,
+                                          float eps, float c1, float c2) {
+  const float a = fmaf(b1, m1, (1.0f - b1) * gi);
+  const float v = fmaf(b2, m2, (1.0f - b2) * gi * gi);
+  m1 = a;
+  m2 = v;
+  const float upd = lr * (a / c1) / (sqrtf(v / c2) + eps);
+  return w - upd;
+}
+
+__global__ void __launch_bounds__(128) adam_kernel(float* w, __nv_bfloat16* wb, const float* part, int splits,
+                                                   float* m1, float* m2, float lr, float b1, float b2, float eps,
+                                                   float c1, float c2) {
+  const int64_t j = 2 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+  if (j >= kP) return;
+  const int64_t i = blockIdx.y * kP + j;
+  const float2 g = partial_sum(part, (int64_t)gridDim.y * kP, splits, i);
+  float2 p = *reinterpret_cast<float2*>(m1 + i), q = *reinterpret_cast<float2*>(m2 + i);
+  float2 u = *reinterpret_cast<float2*>(w + i);
+  u.x = adam_one(u.x, g.x, p.x, q.x, lr, b1, b2, eps, c1, c2);
+  u.y = adam_one(u.y, g.y, p.y, q.y, lr, b1, b2, eps, c1, c2);
+  *reinterpret_cast<float2*>(m1 + i) = p;
+  *reinterpret_cast<float2*>(m2 + i) = q;
+  *reinterpret_cast<float2*>(w + i) = u;
+  *reinterpret_cast<__nv_bfloat162*>(wb + blockIdx.y * kPS + j) = __floats2bfloat162_rn(u.x, u.y);
 }
 
 __global__ void to_bf16_kernel(int64_t total, const float* w, __nv_bfloat16* wb) {
@@ -416,23 +440,27 @@ cudaError_t launch_wgrad(const GradArgs& a, int members, int splits, cudaStream_
   return cudaGetLastError();
 }
 
-__global__ void mlp_grad_reduce_kernel(int64_t total, int splits, const float* part, float* grad) {
-  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-    float acc = part[i];
-    for (int k = 1; k < splits; ++k) acc += part[(int64_t)k * total + i];
-    grad[i] = acc;
-  }
+// pairs of parameters per grid row, 128 threads a block
+constexpr unsigned kPairBlocks = (unsigned)((kP / 2 + 127) / 128);
+static_assert(kP % 2 == 0 && kPS % 2 == 0, "parameter pairs");
+
+__global__ void __launch_bounds__(128) mlp_grad_reduce_kernel(int splits, const float* part, float* grad) {
+  const int64_t j = 2 * (blockIdx.x * (int64_t)blockDim.x + threadIdx.x);
+  if (j >= kP) return;
+  const int64_t i = blockIdx.y * kP + j;
+  const float2 g = partial_sum(part, (int64_t)gridDim.y * kP, splits, i);
+  grad[i] = g.x;   // a caller's array: any float alignment
+  grad[i + 1] = g.y;
 }
 
 cudaError_t launch_grad_reduce(int members, int splits, const float* part, float* grad, cudaStream_t s) {
-  const int64_t total = (int64_t)members * kP;
-  mlp_grad_reduce_kernel<<<grid_1d(total), 256, 0, s>>>(total, splits, part, grad);
+  mlp_grad_reduce_kernel<<<dim3(kPairBlocks, members), 128, 0, s>>>(splits, part, grad);
   return cudaGetLastError();
 }
 
-cudaError_t launch_adam(int64_t total, float* w, __nv_bfloat16* wb, const float* part, int splits, float* m1,
+cudaError_t launch_adam(int members, float* w, __nv_bfloat16* wb, const float* part, int splits, float* m1,
                         float* m2, float lr, float b1, float b2, float eps, float c1, float c2, cudaStream_t s) {
-  adam_kernel<<<grid_1d(total), 256, 0, s>>>(total, w, wb, part, splits, m1, m2, lr, b1, b2, eps, c1, c2);
+  adam_kernel<<<dim3(kPairBlocks, members), 128, 0, s>>>(w, wb, part, splits, m1, m2, lr, b1, b2, eps, c1, c2);
   return cudaGetLastError();
 }
 

@@ -135,10 +135,14 @@ __device__ __forceinline__ void wgrad_fp32_layer(int l, int m, int64_t n, int64_
   }
 }
 
-// batch slices for n samples: one per 128 samples, at most kMaxSplits
+// batch slices for n samples: one per 128 samples, at most kMaxSplits; and the
+// samples of each, a multiple of kChunk
 inline int grad_splits(int64_t n) {
   const int64_t s = (n + 127) / 128;
   return (int)(s < 1 ? 1 : (s > kMaxSplits ? kMaxSplits : s));
+}
+inline int64_t slice_rows(int64_t n, int splits) {
+  return ((n + splits - 1) / splits + kChunk - 1) / kChunk * kChunk;
 }
 
 // Host launchers (the kernels live in mlp.cu).
@@ -149,40 +153,46 @@ cudaError_t launch_backward(const BwdArgs& a, int members, cudaStream_t s);
 cudaError_t launch_wgrad(const GradArgs& a, int members, int splits, cudaStream_t s);
 // grad[m][i] = sum over slices of part[s][m][i], slices in order (deterministic)
 cudaError_t launch_grad_reduce(int members, int splits, const float* part, float* grad, cudaStream_t s);
-// Adam step on the gradient sum over the slice partials part[splits][total]
-cudaError_t launch_adam(int64_t total, float* w, __nv_bfloat16* wb, const float* part, int splits, float* m1,
+// Adam step on the gradient sum over the partials part[splits][members][kP]
+cudaError_t launch_adam(int members, float* w, __nv_bfloat16* wb, const float* part, int splits, float* m1,
                         float* m2, float lr, float b1, float b2, float eps, float c1, float c2, cudaStream_t s);
 cudaError_t launch_to_bf16(int64_t total, const float* w, __nv_bfloat16* wb, cudaStream_t s);
 cudaError_t launch_init(int members, uint64_t seed, float* w, cudaStream_t s);
 cudaError_t launch_gather(int64_t n, const int32_t* idx, const float* x, const float* y, float* xb, float* yb,
                           cudaStream_t s);
 
+// floats of one block of 32 samples x 128 features, with its padding; rows of an
+// array of pairs whose copies start and end on 16 bytes
+constexpr int kBlock = 8 * 516;
+__host__ __device__ constexpr int64_t pair_rows(int64_t n) { return (n + 1) & ~(int64_t)1; }
+
 struct TrainTcArgs {
-  int64_t n;
+  int64_t n;                 // samples of the batch
   int members;
-  const float* x;            // [n][2]
-  const float* y;            // [n][2] targets
+  const float* x;            // [..][2] features
+  const float* y;            // [..][2] targets
+  const int32_t* perm;       // [n] rows of x and y, or null for 0..n-1
   const float* master;       // [members][kP]
   const __nv_bfloat16* wbf;  // [members][kPS]
-  __nv_bfloat16* wbfT;       // [members][3][128][128] W_2..W_4 transposed (written by step 1)
-  float* z;                  // [members][n][4][128] pre-activations
-  float* gp;                 // [members][n][4][128] gelu'(z), written by the forward for the backward
-  float* out;                // [members][n][2]
-  float* dout;               // [members][n][2]
-  float* dz;                 // [members][4][n][128]
-  float* loss;               // [members]
-  float* grad;               // [splits][members][kP] slice partials
-  int64_t rows;              // samples per weight-gradient slice
+  int64_t rows;              // samples per slice
+  int64_t tiles;             // step_tiles(rows, splits)
+  __nv_bfloat16* tile;       // [members][tiles][6][128 * 128] h_1..h_3, dz_4..dz_2 as operand tiles
+  float* block;              // [members][tiles][5][4][kBlock] dz_1..dz_4, gelu(z_4) in blocks of 32 samples
+  float* dout;               // [members][pair_rows(n)][2]
+  float* xb;                 // [pair_rows(n)][2] the batch's features
+  float* loss;               // [members], the per-sample loss sum is added
+  float* grad;               // [splits][members][kP] partial gradients
   unsigned* error;
 };
 
-// tcgen05 training (mlp_tc05_train.cu): step 0 forward (z, out), 1 the
-// transposed weights (wbfT) then loss and input gradients (dout, dz, loss),
-// 2 weight and bias gradients of all five layers into the slice partials.
-cudaError_t launch_train_tc05(int step, const TrainTcArgs& a, int splits, cudaStream_t s);
+// tcgen05 training (mlp_tc05_train.cu): loss and partial gradients of one batch
+int64_t step_tiles(int64_t rows, int splits);
+cudaError_t launch_step_tc05(const TrainTcArgs& a, int splits, int sms, cudaStream_t s);
 
-// tcgen05 screening forward (mlp_tc05.cu): per-member outputs into out
-// [members][n][2], then mean / spread / period-1 probability.
+// tcgen05 forward (mlp_tc05.cu): per-member outputs into out [members][n][2];
+// the screen then reduces them to mean / spread / period-1 probability.
+cudaError_t launch_forward_tc05(int64_t n, int members, const float* x, const float* master, const __nv_bfloat16* wbf,
+                                float* out, unsigned* error, int sms, cudaStream_t s);
 cudaError_t launch_screen_tc05(int64_t n, int members, const float* x, const float* master, const __nv_bfloat16* wbf,
                                float* out, unsigned* error, float* mean, float* stdv, float* p1, int sms,
                                cudaStream_t s);
