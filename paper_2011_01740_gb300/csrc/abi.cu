@@ -19,6 +19,7 @@ cudaError_t launch_ck45(int sys, unsigned flags, const AdaptArgs& a, AdaptLaunch
 cudaError_t launch_ck45_fp32c(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_df(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_df_events(const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
+cudaError_t launch_ck45_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_spt2(int sys, unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_order(const int64_t* steps, int64_t n, int32_t* order, unsigned* hist,
                          cudaStream_t s);
@@ -101,9 +102,11 @@ ens_status cuda_fail(ens_ctx* c, cudaError_t e, const char* what) {
 //   51.7 (160 x 1, longest first), 15,000 45.6 / 52.7, 4,608 frequencies 141.7 /
 //   147.7, split precision 16,384 14.4 / 17.4.
 //   Above that the longest systems bound the run until there are enough
-//   others; FP64 phases want 5 warps per SM (65,536 systems: 57.6, 6 warps
-//   58.9), then 6 (131,044: 207 / 221 at 5), then 12 (262,144: 122 / 149;
-//   524,288: 236 / 295).  Split precision: 8 (131,044: 19.1 / 20.4), 12
+//   others.  FP64 Keller-Miksis phases want 5 teams of three warps per SM (kernel
+//   alone, 131,044 x 4: 110.6, 6 plain warps 126.3; 65,536 x 2: 39.7 / 49.0), then 8
+//   plain warps (200,000 x 2: 78.5, 5 teams 80.3), then 12 (262,144 x 2: 101.9 /
+//   105.1; 524,288: 199 / 209); other FP64 phases 5 warps (65,536: 57.6, 6 warps
+//   58.9), then 6 (131,044: 207 / 221 at 5), then 12.  Split precision: 8 (131,044: 19.1 / 20.4), 12
 //   (262,144: 23.6 / 38.2), 16 (524,288: 37.9 / 74.9), 24 from there.
 //   Double-float phases 4 (65,536: 93.6 / 94.9), then 8 (131,044: 110 / 133;
 //   262,144: 105 / 145).
@@ -113,6 +116,8 @@ ens_status cuda_fail(ens_ctx* c, cudaError_t e, const char* what) {
 //   larger ensembles (262,144: 173 / 211); double-float ones, whose unrolled
 //   trial is bound by instruction fetch, of 8 (131,072: 39.7 / 94.0; 524,288:
 //   138 / 352).
+bool has_teams(const ens_ctx* c);
+
 ens_launch default_launch(const ens_ctx* c) {
   ens_launch L{};
   L.mode = ENS_LAUNCH_PLAIN;
@@ -138,7 +143,9 @@ ens_launch default_launch(const ens_ctx* c) {
   } else if (c->tol.prec == ENS_FP32X2) {
     L.block = per_sm < 640 ? 128 : 256;
   } else if (per_sm < 1300) {
-    L.block = per_sm < 640 ? 160 : 192;
+    L.block = per_sm < 640 || has_teams(c) ? 160 : 192;
+  } else if (per_sm < 1700 && has_teams(c)) {
+    L.block = 256;
   } else {
     L.block = 128;
     L.blocks_per_sm = 3;
@@ -213,12 +220,27 @@ uint64_t timeout_ns(const ens_tol& t) {
   return (uint64_t)(s * 1e9);
 }
 
+// Whether the Keller-Miksis phases of an FP64 launch run in teams of three warps
+// per 32 systems (rkck45_teams.cu): up to 5 teams per SM, which is what the
+// registers hold and where the FP64 pipe still has room (1,073 to 131,044 systems:
+// a seventh to a third faster).  Launches of more warps per SM, chosen where
+// systems abound, keep the one-warp kernel: 524,288 systems 199 ms at 12 warps
+// per SM against 209 ms in 5 teams.
+bool has_teams(const ens_ctx* c) {
+  return c->sys == ENS_SYS_KELLER_MIKSIS && c->tol.n_phases > 0 && c->tol.prec == ENS_FP64 &&
+         c->solver != ENS_RK4 && !(c->km_flags & kKmGeneralExponent);
+}
+bool teams_fit(const ens_ctx* c, AdaptLaunch L) {
+  return has_teams(c) && L.spt == 1 && L.block <= 160 && L.grid * (L.block / 32) <= 5 * (int64_t)c->sm_count;
+}
+
 // the adaptive kernel of the context's precision
 cudaError_t launch_adaptive(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s) {
   if (c->tol.prec == ENS_FP32_COMP) return launch_ck45_fp32c(c->km_flags, a, L, s);
   if (c->tol.prec == ENS_FP32X2)
     return c->sys == ENS_SYS_RELIEF_VALVE ? launch_ck45_df_events(a, L, s) : launch_ck45_df(c->km_flags, a, L, s);
   if (L.spt == 2) return launch_ck45_spt2(c->sys, c->km_flags, a, L, s);
+  if (teams_fit(c, L)) return launch_ck45_teams(c->km_flags, a, L, s);
   return launch_ck45(c->sys, c->km_flags, a, L, s);
 }
 
@@ -590,7 +612,6 @@ ens_status ens_create(ens_ctx** out, ens_system sys, int64_t n, const double* pa
     delete c;
     return ENS_ECUDA;
   }
-  c->launch = default_launch(c);
   st = detect_flags(c);
   if (st != ENS_OK) {
     set_err(nullptr, "%s", c->err);
@@ -598,6 +619,7 @@ ens_status ens_create(ens_ctx** out, ens_system sys, int64_t n, const double* pa
     delete c;
     return st;
   }
+  c->launch = default_launch(c);
   *out = c;
   return ENS_OK;
 }

@@ -17,6 +17,7 @@
 
 namespace ens {
 cudaError_t launch_ck45(int sys, unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
+cudaError_t launch_ck45_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_order(const int64_t* steps, int64_t n, int32_t* order, unsigned* hist, cudaStream_t s);
 void set_call_error(const char* msg);  // text returned by ens_last_error(NULL)
 }  // namespace ens
@@ -182,7 +183,10 @@ extern "C" ens_status ens_solve_noalloc(ens_system sys, int64_t n, const double*
   const int64_t need = (n + 127) / 128;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  if (launch_ck45(sys, flags, a, AdaptLaunch{grid, 128}, s) != cudaSuccess)
+  // four warps of systems per SM: the teams' range (Keller-Miksis with the exponent 21/5)
+  const bool teams = sys == ENS_SYS_KELLER_MIKSIS && !(flags & kKmGeneralExponent);
+  if ((teams ? launch_ck45_teams(flags, a, AdaptLaunch{grid, 128}, s)
+             : launch_ck45(sys, flags, a, AdaptLaunch{grid, 128}, s)) != cudaSuccess)
     return fail(ENS_ECUDA, "ens_solve_noalloc: launch failed");
   return ENS_OK;
 }

@@ -236,6 +236,41 @@ struct KellerMiksis {
   __device__ __forceinline__ void f(double tau, const double* y, double* dy) const {
     fd(drive(tau), tau, y, dy);
   }
+  // accel<double> in parts, the same operations: what does not depend on the
+  // polytropic power g = (1/y1)^(21/5) (early_power) or the drive, and the
+  // rest.  The
+  // paired kernel (rkck45_pairs.cu) has g and the drive computed by another warp.
+  struct Half {
+    double y1, y2, one_c9y2, A, rx, w;
+  };
+  struct Half2 {
+    double b, e, q, yw;
+  };
+  __device__ __forceinline__ double early_power(double y1) const { return polytropic_215(y1, 0.0); }
+  __device__ __forceinline__ Half accel_begin(double y1, double y2) const {
+    const double D = fma(y1, fma(-C9, y2, 1.0), C4C9);
+    const double w = rcp_nr(y1 * D);
+    return {y1, y2, fma(C9, y2, 1.0), fma(C1, y2, C0), D * w, w};
+  }
+  __device__ __forceinline__ Half2 accel_more(const Half& p) const {
+    return {fma(C4, p.y2, C3), fma(C9h, p.y2, 1.5), p.y2 * p.y2, p.y1 * p.w};
+  }
+  __device__ __forceinline__ double accel_mid(const Half& p, const Half2& q, double g) const {   // needs the power,
+    double N = p.A * g;
+    N = fma(-C2, p.one_c9y2, N);
+    N = fma(-q.b, p.rx, N);
+    return fma(-q.e, q.q, N);
+  }
+  __device__ __forceinline__ double accel_last(const Half& p, const Half2& q, double N, double fs, double fc) const {
+    N = fma(-fs, p.one_c9y2, N);   // the drive
+    N = fma(-p.y1, fc, N);
+    return N * q.yw;
+  }
+  __device__ __forceinline__ double accel_at(double y1, double y2, double g, const Drive& d) const {
+    const Half p = accel_begin(y1, y2);
+    const Half2 q = accel_more(p);
+    return accel_last(p, q, accel_mid(p, q, g), d.fs, d.fc);
+  }
 };
 
 // ---------------------------------------------------------------------------

@@ -25,10 +25,10 @@
 // Loops are bounded: max_steps trials per system, 40 event retries in a row,
 // and a wall-clock budget read from %globaltimer; there are no spin-waits.
 #include "common.cuh"
+#include "controller.cuh"
 #include "dual.cuh"
 #include "events.cuh"
 #include "fcmp.cuh"
-#include "rcp_fx.cuh"
 #include "rhs.cuh"
 
 namespace ens {
@@ -144,79 +144,6 @@ __device__ __forceinline__ void pair_trial(const Sys& s, double t, double h, con
   if (PAIR == kDormandPrince) dp_trial(s, t, h, y, k1, y5, err, kn, dn);
   else ck_trial(s, t, h, y, k1, y5, err, dn);
 }
-// right-hand-side evaluations of one trial besides k1
-constexpr uint32_t pair_rhs(int PAIR) { return PAIR == kDormandPrince ? 6u : 5u; }
-
-// E = max_c |err_c| / (atol + rtol max(|y_c|, |y5_c|)), >= 0, or NaN (sign
-// clear) when a trial blew up.  rcp_fx (integer pipe) is within half an ulp
-// plus 2^-57 of 1/sc for the normal sc below 2^1022 of a solve; a zero,
-// subnormal, infinite or NaN sc gives NaN, and a NaN stays the maximum.
-template <int D>
-__device__ __forceinline__ double err_norm(const double* y, const double* y5, const double* err,
-                                           double rtol, double atol) {
-  double E = 0.0;
-#pragma unroll
-  for (int c = 0; c < D; ++c) {
-    const double sc = fma(rtol, nnmax(absd(y[c]), absd(y5[c])), atol);
-    const double r = absd(absd(err[c]) * rcp_fx(sc));
-    E = nnmax(E, r);
-  }
-  return E;
-}
-// accept iff E <= 1 (false for NaN)
-__device__ __forceinline__ bool accept(double E) { return nnbits(E) <= nnbits(1.0); }
-
-// fac = clamp(0.9 E^(-1/5), 0.2, 5).  0.9 E^(-1/5) leaves [0.2, 5] for
-// E > 4.5^5 = 1845.3 and E < 0.18^5 = 1.9e-4, so E is clamped to [1e-4, 2000]
-// first (same result, and keeps the float seed of inv_fifth_root_fx in range).
-// E >= 0 or NaN as err_norm returns it.
-__device__ __forceinline__ double step_factor(double E) {
-  if (nnbits(E) > nnbits(__longlong_as_double(0x7ff0000000000000LL))) return 0.2;  // NaN
-  const double Ec = nnmin(nnmax(E, 1e-4), 2000.0);
-  const double fac = 0.9 * inv_fifth_root_fx(Ec);
-  return nnmin(nnmax(fac, 0.2), 5.0);
-}
-
-// Claim the next system of a persistent lane (or the lane's own system in
-// plain mode).  Returns -1 when no work is left.
-__device__ __forceinline__ int64_t claim(const AdaptArgs& a, bool first) {
-  if (!a.persistent) {
-    if (!first) return -1;
-    const int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    return i < a.n ? i : -1;
-  }
-  const unsigned long long k = atomicAdd(&a.scratch->next, 1ULL);
-  if (k >= (unsigned long long)a.n) return -1;
-  return a.order ? (int64_t)a.order[k] : (int64_t)k;
-}
-
-// First claim of a lane in a persistent, longest-first launch with one block
-// per SM, deterministic and aware of the sub-partitions: warp w of a block
-// runs on sub-partition w mod 4, and a warp that shares its sub-partition
-// gets about half of that sub-partition's FP64 pipe.  The lanes of warps that
-// own their sub-partition take the first ranks of the claim order (the
-// longest systems), the others the next ones; later claims continue from rank
-// gridDim.x * blockDim.x in order (claim_next_after_ranked).  The claim order
-// never changes what a system computes.
-__device__ __forceinline__ int64_t claim_first_by_subpartition(const AdaptArgs& a) {
-  const int W = (int)(blockDim.x >> 5), w = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
-  int u_total = 0, u_before = 0;
-  for (int x = 0; x < W; ++x) {
-    const bool own = ((W - (x & 3) + 3) >> 2) == 1;  // the only warp of block x's sub-partition
-    u_total += own;
-    u_before += own && x < w;
-  }
-  const bool own = ((W - (w & 3) + 3) >> 2) == 1;
-  const int64_t U = (int64_t)gridDim.x * u_total * 32;
-  const int64_t rank = own ? ((int64_t)blockIdx.x * u_total + u_before) * 32 + lane
-                           : U + ((int64_t)blockIdx.x * (W - u_total) + (w - u_before)) * 32 + lane;
-  return rank < a.n ? (int64_t)a.order[rank] : -1;
-}
-__device__ __forceinline__ int64_t claim_next_after_ranked(const AdaptArgs& a) {
-  const unsigned long long k = (unsigned long long)gridDim.x * blockDim.x + atomicAdd(&a.scratch->next, 1ULL);
-  return k < (unsigned long long)a.n ? (int64_t)a.order[k] : -1;
-}
-
 // ---------------------------------------------------------------------------
 // Phase mode (Keller-Miksis, Sec. 4.2): n_phases integrations over
 // tau in [t0, t0 + phase_len] with tau reset at each phase start; running max
@@ -229,7 +156,8 @@ __global__ void __launch_bounds__(256) ck_phased_kernel(AdaptArgs a) {
   constexpr int D = Sys::kDim;
   const double tau_end = a.t0 + a.phase_len;
   const uint64_t deadline = global_ns() + a.timeout_ns;
-  int64_t i = a.first_by_subpartition ? claim_first_by_subpartition(a) : claim(a, true);
+  int64_t i = a.first_by_subpartition ? claim_first_by_subpartition(a, (int)(blockDim.x >> 5))
+                                      : claim(a, true, (int)blockDim.x, (int)threadIdx.x);
   bool timed_out = false;
   Sys s;
   // drive at the phase start (tau = t0), at the current tau, and at tau + h
@@ -356,7 +284,7 @@ __global__ void __launch_bounds__(256) ck_phased_kernel(AdaptArgs a) {
     }
     if (sys_done) {
       finish_system(i);
-      i = a.first_by_subpartition ? claim_next_after_ranked(a) : claim(a, false);
+      i = a.first_by_subpartition ? claim_next_after_ranked(a, (int)blockDim.x) : claim(a, false, 0, 0);
       if (i >= 0) start_system(i);
     }
   }
@@ -431,7 +359,7 @@ __global__ void __launch_bounds__(128) ck_phased2_kernel(AdaptArgs a) {
   // a slot without a first system computes on a copy of system 0 (n > 0)
 #pragma unroll
   for (int q = 0; q < SPT; ++q) {
-    const int64_t k = claim(a, true);
+    const int64_t k = claim(a, true, (int)blockDim.x, (int)threadIdx.x);
     S[q].i = k >= 0 ? k : 0;
     start_system(S[q]);
     S[q].i = k;
@@ -519,7 +447,7 @@ __global__ void __launch_bounds__(128) ck_phased2_kernel(AdaptArgs a) {
       }
       if (sys_done) {
         finish_system(L);
-        L.i = claim(a, false);
+        L.i = claim(a, false, 0, 0);
         if (L.i >= 0) start_system(L);
       }
     }
@@ -550,7 +478,7 @@ __global__ void __launch_bounds__(256) ck_events_kernel(AdaptArgs a) {
   constexpr int D = Sys::kDim;
   const uint64_t deadline = global_ns() + a.timeout_ns;
   const double etol = a.event_tol;
-  int64_t i = claim(a, true);
+  int64_t i = claim(a, true, (int)blockDim.x, (int)threadIdx.x);
   bool timed_out = false;
   Sys s;
   Sys::Drive d5;  // autonomous: empty
@@ -696,7 +624,7 @@ __global__ void __launch_bounds__(256) ck_events_kernel(AdaptArgs a) {
     }
     if (sys_done) {
       finish_system(i);
-      i = claim(a, false);
+      i = claim(a, false, 0, 0);
       if (i >= 0) start_system(i);
     }
   }
@@ -709,7 +637,7 @@ template <class Sys, int PAIR>
 __global__ void __launch_bounds__(256) ck_plain_kernel(AdaptArgs a) {
   constexpr int D = Sys::kDim;
   const uint64_t deadline = global_ns() + a.timeout_ns;
-  int64_t i = claim(a, true);
+  int64_t i = claim(a, true, (int)blockDim.x, (int)threadIdx.x);
   bool timed_out = false;
   Sys s;
   typename Sys::Drive dk, d5;  // drive at t and at t + h
@@ -788,7 +716,7 @@ __global__ void __launch_bounds__(256) ck_plain_kernel(AdaptArgs a) {
     }
     if (sys_done) {
       finish_system(i);
-      i = claim(a, false);
+      i = claim(a, false, 0, 0);
       if (i >= 0) start_system(i);
     }
   }
