@@ -18,6 +18,7 @@ cudaError_t launch_rk4(int sys, bool strict, const Rk4Args& a, int block, int sp
 cudaError_t launch_ck45(int sys, unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_fp32c(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_df(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
+cudaError_t launch_ck45_df_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_df_events(const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_spt2(int sys, unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
@@ -108,14 +109,15 @@ ens_status cuda_fail(ens_ctx* c, cudaError_t e, const char* what) {
 //   105.1; 524,288: 199 / 209); other FP64 phases 5 warps (65,536: 57.6, 6 warps
 //   58.9), then 6 (131,044: 207 / 221 at 5), then 12.  Split precision: 8 (131,044: 19.1 / 20.4), 12
 //   (262,144: 23.6 / 38.2), 16 (524,288: 37.9 / 74.9), 24 from there.
-//   Double-float phases 4 (65,536: 93.6 / 94.9), then 8 (131,044: 110 / 133;
-//   262,144: 105 / 145).
+//   Double-float phases 3 teams of two warps per SM (kernel alone, 65,536 x 4:
+//   72.3, 4 teams 73.9), then 6 (131,044 x 2: 41.9, 4 teams 54.9), then 12 plain
+//   warps (262,144 x 2: 60.8, 8 warps 71.1), then 16 (524,288 x 2: 111.6, 12 120.9).
 //   Valves take about the same number of steps each, and neighbours take them
 //   alike, which claiming by cost breaks up: plain launches of 1 warp a block
 //   (1,000: 21.6 / 25.4; 32,768: 26.4 / 37.2; 65,536: 47.8 / 60.7), of 2 for the
-//   larger ensembles (262,144: 173 / 211); double-float ones, whose unrolled
-//   trial is bound by instruction fetch, of 8 (131,072: 39.7 / 94.0; 524,288:
-//   138 / 352).
+//   larger ensembles (262,144: 173 / 211); double-float ones of 8, whose warps share
+//   the fetch of a long trial (65,536: 20.9, 1 warp a block 21.8; 524,288: 132 /
+//   136; longest first in 5 warps per SM 352).
 bool has_teams(const ens_ctx* c);
 
 ens_launch default_launch(const ens_ctx* c) {
@@ -130,8 +132,7 @@ ens_launch default_launch(const ens_ctx* c) {
     return L;
   }
   if (c->n <= (int64_t)c->sm_count * 128) {
-    // the double-float trial is bound by instruction fetch, which warps of one SM share
-    if (c->tol.prec == ENS_FP32X2) L.block = 128;
+    if (c->tol.prec == ENS_FP32X2) L.block = 64;  // 16,384 x 2: 33.0, one warp a block 35.7
     return L;
   }
   L.mode = ENS_LAUNCH_PERSISTENT;
@@ -141,7 +142,8 @@ ens_launch default_launch(const ens_ctx* c) {
     L.block = per_sm >= 1300 && per_sm < 2600 ? 128 : 256;
     L.blocks_per_sm = per_sm < 1300 ? 1 : per_sm < 2600 ? 3 : per_sm < 5200 ? 2 : 3;
   } else if (c->tol.prec == ENS_FP32X2) {
-    L.block = per_sm < 640 ? 128 : 256;
+    L.block = per_sm < 640 ? 96 : per_sm < 1300 ? 192 : per_sm < 2600 ? 128 : 256;
+    L.blocks_per_sm = per_sm < 1300 ? 1 : per_sm < 2600 ? 3 : 2;
   } else if (per_sm < 1300) {
     L.block = per_sm < 640 || has_teams(c) ? 160 : 192;
   } else if (per_sm < 1700 && has_teams(c)) {
@@ -234,11 +236,20 @@ bool teams_fit(const ens_ctx* c, AdaptLaunch L) {
   return has_teams(c) && L.spt == 1 && L.block <= 160 && L.grid * (L.block / 32) <= 5 * (int64_t)c->sm_count;
 }
 
+// The same for double-float phases, in teams of two (df64.cu): up to 6 per SM
+// (131,044 systems x 2 periods 41.9 ms against 45.4 in plain warps; 262,144 x 2
+// 83.7 against 62.1 in 12 plain warps per SM).
+bool df_teams_fit(const ens_ctx* c, AdaptLaunch L) {
+  return L.block <= 192 && L.grid * (L.block / 32) <= 6 * (int64_t)c->sm_count;
+}
+
 // the adaptive kernel of the context's precision
 cudaError_t launch_adaptive(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s) {
   if (c->tol.prec == ENS_FP32_COMP) return launch_ck45_fp32c(c->km_flags, a, L, s);
-  if (c->tol.prec == ENS_FP32X2)
-    return c->sys == ENS_SYS_RELIEF_VALVE ? launch_ck45_df_events(a, L, s) : launch_ck45_df(c->km_flags, a, L, s);
+  if (c->tol.prec == ENS_FP32X2) {
+    if (c->sys == ENS_SYS_RELIEF_VALVE) return launch_ck45_df_events(a, L, s);
+    return df_teams_fit(c, L) ? launch_ck45_df_teams(c->km_flags, a, L, s) : launch_ck45_df(c->km_flags, a, L, s);
+  }
   if (L.spt == 2) return launch_ck45_spt2(c->sys, c->km_flags, a, L, s);
   if (teams_fit(c, L)) return launch_ck45_teams(c->km_flags, a, L, s);
   return launch_ck45(c->sys, c->km_flags, a, L, s);

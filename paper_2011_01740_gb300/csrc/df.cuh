@@ -42,21 +42,44 @@ __host__ __device__ __forceinline__ float fma_f(float a, float b, float c) {
 #endif
 }
 
+// operations that the device compiler may not contract into an FMA
+__host__ __device__ __forceinline__ float add_f(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fadd_rn(a, b);
+#else
+  return a + b;
+#endif
+}
+__host__ __device__ __forceinline__ float sub_f(float a, float b) { return add_f(a, -b); }
+__host__ __device__ __forceinline__ float mul_f(float a, float b) {
+#ifdef __CUDA_ARCH__
+  return __fmul_rn(a, b);
+#else
+  return a * b;
+#endif
+}
+
 // error-free transformations
 __host__ __device__ __forceinline__ DF fast_two_sum(float a, float b) {  // requires |a| >= |b| (or a == 0)
-  const float s = a + b;
-  const float z = s - a;
-  return {s, b - z};
+  const float s = add_f(a, b);
+  const float z = sub_f(s, a);
+  return {s, sub_f(b, z)};
 }
 __host__ __device__ __forceinline__ DF two_sum(float a, float b) {
-  const float s = a + b;
-  const float ap = s - b;
-  const float bp = s - ap;
-  return {s, (a - ap) + (b - bp)};
+  const float s = add_f(a, b);
+  const float ap = sub_f(s, b);
+  const float bp = sub_f(s, ap);
+  return {s, add_f(sub_f(a, ap), sub_f(b, bp))};
 }
 __host__ __device__ __forceinline__ DF two_prod(float a, float b) {
-  const float p = a * b;
+  const float p = mul_f(a, b);
   return {p, fma_f(a, b, -p)};
+}
+// a + b c with the product in FMAs, for |a| >= |b c|
+__host__ __device__ __forceinline__ DF fast_two_sum_fma(float a, float b, float c) {
+  const float s = fma_f(b, c, a);
+  const float z = sub_f(s, a);
+  return {s, fma_f(b, c, -z)};
 }
 
 __host__ __device__ __forceinline__ DF make(float x) { return {x, 0.0f}; }
@@ -66,9 +89,9 @@ __host__ __device__ __forceinline__ DF neg(DF x) { return {-x.hi, -x.lo}; }
 __host__ __device__ __forceinline__ DF add(DF x, DF y) {
   const DF s = two_sum(x.hi, y.hi);
   const DF t = two_sum(x.lo, y.lo);
-  const float c = s.lo + t.hi;
+  const float c = add_f(s.lo, t.hi);
   const DF v = fast_two_sum(s.hi, c);
-  const float w = t.lo + v.lo;
+  const float w = add_f(t.lo, v.lo);
   return fast_two_sum(v.hi, w);
 }
 __host__ __device__ __forceinline__ DF sub(DF x, DF y) { return add(x, neg(y)); }
@@ -82,12 +105,12 @@ __host__ __device__ __forceinline__ DF sub(DF x, DF y) { return add(x, neg(y)); 
 // result even under cancellation.
 __host__ __device__ __forceinline__ DF add_terms(DF x, DF y) {
   const DF s = two_sum(x.hi, y.hi);
-  return fast_two_sum(s.hi, s.lo + (x.lo + y.lo));
+  return fast_two_sum(s.hi, add_f(s.lo, add_f(x.lo, y.lo)));
 }
 // DW + FP (10 flops)
 __host__ __device__ __forceinline__ DF add(DF x, float y) {
   const DF s = two_sum(x.hi, y);
-  const float v = x.lo + s.lo;
+  const float v = add_f(x.lo, s.lo);
   return fast_two_sum(s.hi, v);
 }
 
@@ -101,10 +124,10 @@ __host__ __device__ __forceinline__ DF mul(DF x, float y) {
 // DW x DW (9 flops)
 __host__ __device__ __forceinline__ DF mul(DF x, DF y) {
   const DF c = two_prod(x.hi, y.hi);
-  const float tl0 = x.lo * y.lo;
+  const float tl0 = mul_f(x.lo, y.lo);
   const float tl1 = fma_f(x.hi, y.lo, tl0);
   const float cl2 = fma_f(x.lo, y.hi, tl1);
-  return fast_two_sum(c.hi, c.lo + cl2);
+  return fast_two_sum(c.hi, add_f(c.lo, cl2));
 }
 
 // a b + c
@@ -122,8 +145,8 @@ __host__ __device__ __forceinline__ DF rcp(DF y) {
   const float r0 = 1.0f / y.hi;
 #endif
   const DF p = mul(y, r0);                       // y r0 = 1 - e
-  const float e = (1.0f - p.hi) - p.lo;          // 1 - p.hi is exact (Sterbenz)
-  return fast_two_sum(r0, r0 * fma_f(e, e, e));  // r0 (1 + e + e^2): error about e^3
+  const float e = sub_f(sub_f(1.0f, p.hi), p.lo);  // 1 - p.hi is exact (Sterbenz)
+  return fast_two_sum_fma(r0, r0, fma_f(e, e, e));  // r0 (1 + e + e^2): error about e^3
 }
 
 // x^(-1/5) for x > 0: float seed v (about 22 correct bits), residual
@@ -142,7 +165,13 @@ __host__ __device__ __forceinline__ DF inv_fifth_root(DF x) {
   const DF v5 = mul(v4, v);
   const DF xv5 = mul(x, v5);
   const DF r = add(neg(xv5), 1.0f);                          // about 1e-6
-  const DF c = add(DF{0.2f, -2.98023224e-09f}, 0.12f * r.hi);   // 1/5 (as a pair) + 3 r / 25
+  // 1/5 (as a pair) + 3 r / 25: two_sum(0.2, b) with b = 0.12 r, its error term
+  // taken from the unrounded product
+  const float b = mul_f(0.12f, r.hi);
+  const float s = add_f(0.2f, b);
+  const float ap = sub_f(s, b), bp = sub_f(s, ap);
+  const float e = add_f(sub_f(0.2f, ap), fma_f(0.12f, r.hi, -bp));
+  const DF c = fast_two_sum(s, add_f(-2.98023224e-09f, e));
   return add(make(v), mul(mul(r, c), v));
 }
 
@@ -163,8 +192,8 @@ __host__ __device__ __forceinline__ DF sqrt(DF x) {
   const float inv2 = 0.5f / s0;
 #endif
   const DF p = two_prod(s0, s0);
-  const float r = ((x.hi - p.hi) - p.lo) + x.lo;
-  return fast_two_sum(s0, r * inv2);
+  const float r = add_f(sub_f(sub_f(x.hi, p.hi), p.lo), x.lo);
+  return fast_two_sum_fma(s0, r, inv2);
 }
 
 // double <-> double-word through the integer pipe (a conversion instruction
@@ -250,6 +279,105 @@ __host__ __device__ __forceinline__ DF from_double_sub(double x) {
 }
 // double-word -> double: one FP64 addition
 __host__ __device__ __forceinline__ double to_double(DF x) { return widen(x.hi) + widen(x.lo); }
+
+// ---------------------------------------------------------------------------
+// Two double-floats side by side, on the packed FP32 instructions (two lanes per
+// instruction): each half of every operation below is the scalar one above, in
+// the same order, so the results are the same bits.
+// ---------------------------------------------------------------------------
+#ifdef __CUDACC__
+typedef unsigned long long F2;  // two floats, the first in the low half
+#else
+struct F2 {
+  float x, y;
+};
+#endif
+__host__ __device__ __forceinline__ F2 f2(float x, float y) {
+#ifdef __CUDACC__
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(x), "f"(y));
+  return r;
+#else
+  return {x, y};
+#endif
+}
+__host__ __device__ __forceinline__ void unpack(F2 a, float* x, float* y) {
+#ifdef __CUDACC__
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(*x), "=f"(*y) : "l"(a));
+#else
+  *x = a.x, *y = a.y;
+#endif
+}
+__host__ __device__ __forceinline__ F2 add_f(F2 a, F2 b) {
+#ifdef __CUDACC__
+  F2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+#else
+  return {a.x + b.x, a.y + b.y};
+#endif
+}
+__host__ __device__ __forceinline__ F2 mul_f(F2 a, F2 b) {
+#ifdef __CUDACC__
+  F2 r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+#else
+  return {a.x * b.x, a.y * b.y};
+#endif
+}
+__host__ __device__ __forceinline__ F2 fma_f(F2 a, F2 b, F2 c) {
+#ifdef __CUDACC__
+  F2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+#else
+  return {fma_f(a.x, b.x, c.x), fma_f(a.y, b.y, c.y)};
+#endif
+}
+// a - b as one fused multiply-add, a + b (-1): the same rounding
+__host__ __device__ __forceinline__ F2 sub_f(F2 a, F2 b) { return fma_f(b, f2(-1.0f, -1.0f), a); }
+
+struct DF2 {
+  F2 hi, lo;
+};
+__host__ __device__ __forceinline__ DF2 pack(DF a, DF b) { return {f2(a.hi, b.hi), f2(a.lo, b.lo)}; }
+__host__ __device__ __forceinline__ DF2 both(DF a) { return pack(a, a); }
+__host__ __device__ __forceinline__ void unpack(DF2 v, DF* a, DF* b) {
+  unpack(v.hi, &a->hi, &b->hi);
+  unpack(v.lo, &a->lo, &b->lo);
+}
+__host__ __device__ __forceinline__ DF2 fast_two_sum(F2 a, F2 b) {
+  const F2 s = add_f(a, b);
+  return {s, sub_f(b, sub_f(s, a))};
+}
+__host__ __device__ __forceinline__ DF2 two_sum(F2 a, F2 b) {
+  const F2 s = add_f(a, b);
+  const F2 ap = sub_f(s, b);
+  const F2 bp = sub_f(s, ap);
+  return {s, add_f(sub_f(a, ap), sub_f(b, bp))};
+}
+__host__ __device__ __forceinline__ DF2 add(DF2 x, DF2 y) {
+  const DF2 s = two_sum(x.hi, y.hi);
+  const DF2 t = two_sum(x.lo, y.lo);
+  const DF2 v = fast_two_sum(s.hi, add_f(s.lo, t.hi));
+  return fast_two_sum(v.hi, add_f(t.lo, v.lo));
+}
+__host__ __device__ __forceinline__ DF2 add_terms(DF2 x, DF2 y) {
+  const DF2 s = two_sum(x.hi, y.hi);
+  return fast_two_sum(s.hi, add_f(s.lo, add_f(x.lo, y.lo)));
+}
+// x y with nh = -x.hi given: p = x.hi y.hi appears as -p = nh y.hi
+__host__ __device__ __forceinline__ DF2 mul(DF2 x, F2 nh, DF2 y) {
+  const F2 np = mul_f(nh, y.hi);
+  const F2 e = fma_f(x.hi, y.hi, np);
+  const F2 tl0 = mul_f(x.lo, y.lo);
+  const F2 cl2 = fma_f(x.lo, y.hi, fma_f(x.hi, y.lo, tl0));
+  const F2 c = add_f(e, cl2);
+  const F2 s = sub_f(c, np);
+  return {s, sub_f(c, add_f(s, np))};
+}
+__host__ __device__ __forceinline__ DF2 mul(DF2 x, DF2 y) { return mul(x, mul_f(x.hi, f2(-1.0f, -1.0f)), y); }
 
 // ordering of normalised pairs
 __host__ __device__ __forceinline__ bool gt(DF a, DF b) { return a.hi > b.hi || (a.hi == b.hi && a.lo > b.lo); }

@@ -41,6 +41,7 @@
 // ENS_SYS_TIMEOUT, and a helper whose wait expires leaves.
 #include "common.cuh"
 #include "controller.cuh"
+#include "mailbox.cuh"
 #include "rhs.cuh"
 
 namespace ens {
@@ -48,7 +49,6 @@ namespace ens {
 namespace {
 
 constexpr int kMaxTeams = 5;             // teams of three warps per block
-constexpr uint32_t kTeamWait = 1u << 24; // polls of one wait
 
 // barriers of a team's mailbox
 enum : int { kReq = 0, kRsp = 2, kCtlReq = 4, kCtlRsp = 5, kStart = 6, kDrive = 7, kBars = 12 };
@@ -64,33 +64,6 @@ struct __align__(16) Mailbox {
   int run;                     // 0: no systems left
   unsigned long long bar[kBars];
 };
-
-__device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-// the warp's writes above are complete for whoever waits for this phase
-__device__ __forceinline__ void post(unsigned long long* bar) {
-  __syncwarp();
-  if ((threadIdx.x & 31) == 0)
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-
-// wait for the next phase; `phase` is that barrier's phase count in this warp
-__device__ __forceinline__ bool await(unsigned long long* bar, uint32_t& phase) {
-  const uint32_t b = smem_addr(bar), parity = phase & 1u;
-  ++phase;
-  for (uint32_t k = 0; k < kTeamWait; ++k) {
-    uint32_t done;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}\n"
-        : "=r"(done)
-        : "r"(b), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
 
 // stage times of stages 2..6 in steps (a stage at t + h is fma(1, h, t), the same bits)
 template <int PAIR>
@@ -441,10 +414,7 @@ template <class Sys, int PAIR>
 __global__ void __launch_bounds__(96 * kMaxTeams) ck_phased_teams_kernel(AdaptArgs a) {
   __shared__ Mailbox boxes[kMaxTeams];
   const int W = (int)blockDim.x / 96, w = (int)(threadIdx.x >> 5);
-  if (threadIdx.x < (unsigned)W) {
-    for (int k = 0; k < kBars; ++k)
-      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(&boxes[threadIdx.x].bar[k])));
-  }
+  if (threadIdx.x < (unsigned)W) init_bars(boxes[threadIdx.x].bar, kBars);
   __syncthreads();
   if (w < W) main_warp<Sys, PAIR>(a, boxes[w], W);
   else if (w < 2 * W) power_warp<Sys>(a, boxes[w - W]);

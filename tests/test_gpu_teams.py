@@ -1,5 +1,5 @@
-"""The Keller-Miksis kernel with teams of three warps gives the bits of the
-one-warp kernel: at the edges of its warps and blocks, for both pairs and one or
+"""The Keller-Miksis kernels with teams of warps (FP64: three, double-float: two)
+give the bits of the one-warp kernels: at the edges of its warps and blocks, for both pairs and one or
 two frequencies, with a phase that does not start at tau = 0 or last one period
 (the drive then differs between a phase's end and the next one's start), and for
 systems that are retired early."""
@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 READ = (ens.ENS_STATE, ens.ENS_ACC, ens.ENS_STATUS, ens.ENS_NSTEPS, ens.ENS_NREJ, ens.ENS_NRHS, ens.ENS_TIME,
         ens.ENS_DT)
 PLAIN, PERSISTENT = ens.ENS_LAUNCH_PLAIN, ens.ENS_LAUNCH_PERSISTENT
-ONE_WARP = dict(mode=PLAIN, block=192, blocks_per_sm=0)        # blocks above 160 threads: no teams
+ONE_WARP = dict(mode=PLAIN, block=256, blocks_per_sm=0)        # blocks above 160 (192) threads: no teams
 
 
 def _solve(ctx, **launch):
@@ -55,10 +55,23 @@ def test_teams_give_the_one_warp_bits(n, launch, solver, dual):
     _compare(n, launch, solver=solver, dual=dual)
 
 
+@pytest.mark.parametrize("dual", [False, True])
+@pytest.mark.parametrize("n,launch", [
+    (1, dict(mode=PLAIN, block=32, blocks_per_sm=0)),
+    (193, dict(mode=PLAIN, block=192, blocks_per_sm=0)),
+    (23000, dict(mode=PERSISTENT, block=128, blocks_per_sm=1, cost_order=0)),
+    (60000, dict(mode=PERSISTENT, block=192, blocks_per_sm=1, cost_order=1)),
+    (30000, dict(mode=PERSISTENT, block=64, blocks_per_sm=3, cost_order=1)),
+])
+def test_double_float_teams_give_the_one_warp_bits(n, launch, dual):
+    _compare(n, launch, dual=dual, prec=ens.ENS_FP32X2)
+
+
 SMALL = dict(mode=PERSISTENT, block=64, blocks_per_sm=1, cost_order=1)
 
 
-@pytest.mark.parametrize("solver", [ens.ENS_RKCK45, ens.ENS_DOPRI5])
+@pytest.mark.parametrize("solver,prec", [(ens.ENS_RKCK45, ens.ENS_FP64), (ens.ENS_DOPRI5, ens.ENS_FP64),
+                                         (ens.ENS_RKCK45, ens.ENS_FP32X2)])
 @pytest.mark.parametrize("kw", [
     dict(t0=0.3, phase_len=0.7),                       # the phase start's drive has other bits than its end's
     dict(n_phases=5, n_transient=4),
@@ -66,20 +79,21 @@ SMALL = dict(mode=PERSISTENT, block=64, blocks_per_sm=1, cost_order=1)
     dict(dt_min=3e-3, dt0=0.1),                        # step-size underflow after a rejection
     dict(rtol=1e-4, atol=1e-4, dt0=0.5, dt_max=0.5),   # many rejections
 ])
-def test_teams_keep_phases_budgets_and_rejections(kw, solver):
-    ref = _compare(700, SMALL, solver=solver, **kw)
+def test_teams_keep_phases_budgets_and_rejections(kw, solver, prec):
+    ref = _compare(700, SMALL, solver=solver, prec=prec, **kw)
     if "max_steps" in kw or "dt_min" in kw:
         assert ref[0] == ens.ENS_ESYSTEM
 
 
-def test_teams_stop_at_the_wall_clock_budget():
+@pytest.mark.parametrize("prec", [ens.ENS_FP64, ens.ENS_FP32X2])
+def test_teams_stop_at_the_wall_clock_budget(prec):
     """Systems that a 1 us budget catches are flagged; the call returns and says so."""
     n = 700
     km = W.km(1, n, pa_max=1e5)
     ph = km["phys"]
     C = ens.ens_km_coefficients(*[ph[k] for k in ("pA1", "f1", "pA2", "f2", "theta", "RE")], km["liquid"])
     ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS, n, C, km["y0"], (0.0, 1.0), ens.ENS_RKCK45,
-                         ens.make_tol(n_phases=64, timeout_s=1e-6))
+                         ens.make_tol(n_phases=64, timeout_s=1e-6, prec=prec))
     try:
         got = _solve(ctx, mode=PLAIN, block=32, blocks_per_sm=0)
     finally:
