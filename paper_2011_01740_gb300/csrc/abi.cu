@@ -114,10 +114,10 @@ ens_status cuda_fail(ens_ctx* c, cudaError_t e, const char* what) {
 //   warps (262,144 x 2: 60.8, 8 warps 71.1), then 16 (524,288 x 2: 111.6, 12 120.9).
 //   Valves take about the same number of steps each, and neighbours take them
 //   alike, which claiming by cost breaks up: plain launches of 1 warp a block
-//   (1,000: 21.6 / 25.4; 32,768: 26.4 / 37.2; 65,536: 47.8 / 60.7), of 2 for the
-//   larger ensembles (262,144: 173 / 211); double-float ones of 8, whose warps share
-//   the fetch of a long trial (65,536: 20.9, 1 warp a block 21.8; 524,288: 132 /
-//   136; longest first in 5 warps per SM 352).
+//   (1,000: 21.5 / 25.4; 32,768: 25.8 / 37.2; 65,536: 46.4 / 60.7; 262,144: 168 /
+//   211; 2 warps a block 21.4, 28.2, 46.7 and 170); double-float ones of 8, whose
+//   warps share the fetch of a long trial (65,536: 20.8, 1 warp a block 21.8; 524,288:
+//   132 / 136; persistent 5 warps per SM 282).
 bool has_teams(const ens_ctx* c);
 
 ens_launch default_launch(const ens_ctx* c) {
@@ -128,7 +128,6 @@ ens_launch default_launch(const ens_ctx* c) {
   if (c->solver == ENS_RK4) return L;
   if (c->sys == ENS_SYS_RELIEF_VALVE && c->tol.n_phases == 0) {
     if (c->tol.prec == ENS_FP32X2) L.block = 256;
-    else if (per_sm >= 512) L.block = 64;
     return L;
   }
   if (c->n <= (int64_t)c->sm_count * 128) {

@@ -5,6 +5,7 @@
 #include "common.cuh"
 #include "fcmp.cuh"
 #include "fifth_root_fx.cuh"
+#include "fp64ops.cuh"
 #include "rcp_fx.cuh"
 
 namespace ens {
@@ -23,7 +24,7 @@ __device__ __forceinline__ double err_norm(const double* y, const double* y5, co
 #pragma unroll
   for (int c = 0; c < D; ++c) {
     const double sc = fma(rtol, nnmax(absd(y[c]), absd(y5[c])), atol);
-    const double r = absd(absd(err[c]) * rcp_fx(sc));
+    const double r = absd(fmul(absd(err[c]), rcp_fx(sc)));
     E = nnmax(E, r);
   }
   return E;
@@ -38,7 +39,7 @@ __device__ __forceinline__ bool accept(double E) { return nnbits(E) <= nnbits(1.
 __device__ __forceinline__ double step_factor(double E) {
   if (nnbits(E) > nnbits(__longlong_as_double(0x7ff0000000000000LL))) return 0.2;  // NaN
   const double Ec = nnmin(nnmax(E, 1e-4), 2000.0);
-  const double fac = 0.9 * inv_fifth_root_fx(Ec);
+  const double fac = fmul(0.9, inv_fifth_root_fx(Ec));
   return nnmin(nnmax(fac, 0.2), 5.0);
 }
 

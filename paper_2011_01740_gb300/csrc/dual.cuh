@@ -30,6 +30,7 @@ __device__ __forceinline__ Dual& operator-=(Dual& a, Dual b) {
 // (a b)' = a' b + a b'
 __device__ __forceinline__ Dual operator*(Dual a, Dual b) { return {a.v * b.v, fma(a.d, b.v, a.v * b.d)}; }
 __device__ __forceinline__ Dual operator*(double a, Dual b) { return {a * b.v, a * b.d}; }
+__device__ __forceinline__ Dual fmul(Dual a, Dual b) { return a * b; }
 
 // fma(a, b, c) = a b + c: derivative a' b + a b' + c'
 __device__ __forceinline__ Dual fma(Dual a, Dual b, Dual c) {

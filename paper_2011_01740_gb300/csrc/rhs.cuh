@@ -11,6 +11,7 @@
 
 #include "common.cuh"
 #include "fifth_root_fx.cuh"
+#include "fp64ops.cuh"
 #include "sincos_fx.cuh"
 #include "sqrt_fx.cuh"
 
@@ -210,8 +211,8 @@ struct KellerMiksis {
     // one reciprocal serves both 1/y1 and 1/D: w = 1 / (y1 D), 1/y1 = D w, N/D = N y1 w;
     // D = y1 (1 - C9 y2) + C4 C9
     const T D = fma(y1, fma(-C9, y2, 1.0), C4C9);
-    const T w = rcp_nr(y1 * D);
-    const T rx = D * w;
+    const T w = rcp_nr(fmul(y1, D));
+    const T rx = fmul(D, w);
     T g;
     if (EXP215) {
       g = polytropic_215(y1, rx);
@@ -219,14 +220,14 @@ struct KellerMiksis {
       g = pow(rx, C10);
     }
     const T one_c9y2 = fma(C9, y2, 1.0);
-    T N = fma(C1, y2, C0) * g;
+    T N = fmul(fma(C1, y2, C0), g);
     N = fma(-C2, one_c9y2, N);
     N = fma(-fma(C4, y2, C3), rx, N);
     // - (1 - C9 y2 / 3) * 1.5 * y2^2 = - (1.5 - 0.5 C9 y2) y2^2
-    N = fma(-fma(C9h, y2, 1.5), y2 * y2, N);
+    N = fma(-fma(C9h, y2, 1.5), fmul(y2, y2), N);
     N = fma(-d.fs, one_c9y2, N);
     N = fma(-y1, d.fc, N);
-    return N * (y1 * w);
+    return fmul(N, fmul(y1, w));
   }
   __device__ __forceinline__ void fd(const Drive& d, double tau, const double* y, double* dy) const {
     (void)tau;
@@ -297,9 +298,9 @@ struct ReliefValve {
   __device__ __forceinline__ void f(double t, const double* y, double* dy) const {
     (void)t;
     dy[0] = y[1];
-    dy[1] = fma(-kappa, y[1], y[2] - (y[0] + delta));
+    dy[1] = fma(-kappa, y[1], fsub(y[2], fadd(y[0], delta)));
     const double y3 = __double2hiint(y[2]) < 0 ? 0.0 : y[2];
-    dy[2] = beta * fma(-y[0], sqrt_fx(y3), q);
+    dy[2] = fmul(beta, fma(-y[0], sqrt_fx(y3), q));
   }
   using Drive = NoDrive;
   __device__ __forceinline__ Drive drive(double) const { return {}; }
