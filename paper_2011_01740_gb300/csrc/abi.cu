@@ -21,6 +21,7 @@ cudaError_t launch_ck45_df(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cu
 cudaError_t launch_ck45_df_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_df_events(const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
+cudaError_t launch_ck45_relay(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_spt2(int sys, unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_order(const int64_t* steps, int64_t n, int32_t* order, unsigned* hist,
                          cudaStream_t s);
@@ -235,6 +236,14 @@ bool teams_fit(const ens_ctx* c, AdaptLaunch L) {
   return has_teams(c) && L.spt == 1 && L.block <= 160 && L.grid * (L.block / 32) <= 5 * (int64_t)c->sm_count;
 }
 
+// Whether they run in relays (rkck45_relay.cu): blocks of one warp of systems, up to
+// two per SM, which is what the registers hold.  Up to there the longest system
+// bounds the run, and its trial takes two thirds of the teams' time (1 system 30.3 /
+// 19.5 ms, 9,700 x 2 periods 32.6 / 21.9).
+bool relay_fits(const ens_ctx* c, AdaptLaunch L) {
+  return has_teams(c) && L.spt == 1 && L.block == 32 && L.grid <= 2 * (int64_t)c->sm_count;
+}
+
 // The same for double-float phases, in teams of two (df64.cu): up to 6 per SM
 // (131,044 systems x 2 periods 41.9 ms against 45.4 in plain warps; 262,144 x 2
 // 83.7 against 62.1 in 12 plain warps per SM).
@@ -250,6 +259,7 @@ cudaError_t launch_adaptive(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L,
     return df_teams_fit(c, L) ? launch_ck45_df_teams(c->km_flags, a, L, s) : launch_ck45_df(c->km_flags, a, L, s);
   }
   if (L.spt == 2) return launch_ck45_spt2(c->sys, c->km_flags, a, L, s);
+  if (relay_fits(c, L)) return launch_ck45_relay(c->km_flags, a, L, s);
   if (teams_fit(c, L)) return launch_ck45_teams(c->km_flags, a, L, s);
   return launch_ck45(c->sys, c->km_flags, a, L, s);
 }

@@ -17,15 +17,18 @@ constexpr uint32_t pair_rhs(int PAIR) { return PAIR == kDormandPrince ? 6u : 5u;
 // clear) when a trial blew up.  rcp_fx (integer pipe) is within half an ulp
 // plus 2^-57 of 1/sc for the normal sc below 2^1022 of a solve; a zero,
 // subnormal, infinite or NaN sc gives NaN, and a NaN stays the maximum.
+// (1 / sc and the ratio on their own: err_weight, err_ratio)
+__device__ __forceinline__ double err_weight(double y, double y5, double rtol, double atol) {
+  return rcp_fx(fma(rtol, nnmax(absd(y), absd(y5)), atol));
+}
+__device__ __forceinline__ double err_ratio(double err, double weight) { return absd(fmul(absd(err), weight)); }
 template <int D>
 __device__ __forceinline__ double err_norm(const double* y, const double* y5, const double* err,
                                            double rtol, double atol) {
   double E = 0.0;
 #pragma unroll
   for (int c = 0; c < D; ++c) {
-    const double sc = fma(rtol, nnmax(absd(y[c]), absd(y5[c])), atol);
-    const double r = absd(fmul(absd(err[c]), rcp_fx(sc)));
-    E = nnmax(E, r);
+    E = nnmax(E, err_ratio(err[c], err_weight(y[c], y5[c], rtol, atol)));
   }
   return E;
 }

@@ -1,4 +1,4 @@
-// mailbox.cuh -- messages between the warps of a team (rkck45_teams.cu, df64.cu):
+// mailbox.cuh -- messages between the warps of a team (rkck45_teams.cu, rkck45_relay.cu, df64.cu):
 // a warp's lanes write to shared memory and one of them arrives on an mbarrier,
 // whose phase the receiving warp awaits.  Waits are bounded.
 #pragma once
@@ -36,9 +36,12 @@ __device__ __forceinline__ bool await(unsigned long long* bar, uint32_t& phase) 
   return false;
 }
 
+// a barrier whose phases end when `senders` warps have posted
+__device__ __forceinline__ void init_bar(unsigned long long* bar, int senders) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(senders));
+}
 __device__ __forceinline__ void init_bars(unsigned long long* bar, int count) {
-  for (int k = 0; k < count; ++k)
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_addr(bar + k)));
+  for (int k = 0; k < count; ++k) init_bar(bar + k, 1);
 }
 
 }  // namespace ens

@@ -18,6 +18,7 @@
 namespace ens {
 cudaError_t launch_ck45(int sys, unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
+cudaError_t launch_ck45_relay(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_order(const int64_t* steps, int64_t n, int32_t* order, unsigned* hist, cudaStream_t s);
 void set_call_error(const char* msg);  // text returned by ens_last_error(NULL)
 }  // namespace ens
@@ -183,10 +184,13 @@ extern "C" ens_status ens_solve_noalloc(ens_system sys, int64_t n, const double*
   const int64_t need = (n + 127) / 128;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  // four warps of systems per SM: the teams' range (Keller-Miksis with the exponent 21/5)
+  // Keller-Miksis with the exponent 21/5: relays up to two warps of systems per SM (1,073
+  // x 2 periods 33 -> 21 ms), else teams, whose range ends at five
   const bool teams = sys == ENS_SYS_KELLER_MIKSIS && !(flags & kKmGeneralExponent);
-  if ((teams ? launch_ck45_teams(flags, a, AdaptLaunch{grid, 128}, s)
-             : launch_ck45(sys, flags, a, AdaptLaunch{grid, 128}, s)) != cudaSuccess)
+  const bool relay = teams && n <= 64 * (int64_t)sms;
+  if ((relay   ? launch_ck45_relay(flags, a, AdaptLaunch{(n + 31) / 32, 32}, s)
+       : teams ? launch_ck45_teams(flags, a, AdaptLaunch{grid, 128}, s)
+               : launch_ck45(sys, flags, a, AdaptLaunch{grid, 128}, s)) != cudaSuccess)
     return fail(ENS_ECUDA, "ens_solve_noalloc: launch failed");
   return ENS_OK;
 }

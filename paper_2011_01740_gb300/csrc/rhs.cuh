@@ -168,6 +168,7 @@ struct NoDrive {};
 // ---------------------------------------------------------------------------
 template <bool DUAL, bool EXP215 = false>
 struct KellerMiksis {
+  static constexpr bool kDual = DUAL;
   static constexpr int kDim = 2;
   static constexpr int kPar = 13;
   static constexpr int kPhaseRows = 0;

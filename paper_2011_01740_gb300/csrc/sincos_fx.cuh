@@ -77,6 +77,37 @@ __host__ __device__ __forceinline__ constexpr uint64_t kQ(int k) {
 
 }  // namespace fx
 
+// The two polynomials of sincos2pi_fx on their own: with SIN that of the sine of
+// the reduced argument, else that of its cosine.  Either gives the sine or the
+// cosine of 2 pi x, which depends on the quarter turn (*sine); the bits are those
+// of sincos2pi_fx.
+template <bool SIN>
+__host__ __device__ __forceinline__ double sincos2pi_half(double x, bool* sine) {
+  using namespace fx;
+  const uint64_t b = dbits(x);
+  const bool finite = ((b >> 52) & 0x7ff) != 0x7ff;
+  const uint64_t F = turns(b) + (1ull << 61);
+  const unsigned q = (unsigned)(F >> 62);
+  const uint64_t W = ((F & 0x3fffffffffffffffull) - (1ull << 61)) << 2;
+  const bool neg = (W >> 63) != 0;
+  const uint64_t A = neg ? (uint64_t)0 - W : W;
+  const uint64_t V = mulhi(A, A);
+  uint64_t p = SIN ? kS(9) : kQ(8), z;
+#pragma unroll
+  for (int k = SIN ? 8 : 7; k >= 0; --k) p = (SIN ? kS(k) : kQ(k)) - mulhi(V, p);
+  if (SIN) {
+    const uint64_t sa = mulhi(A, p) << 1;
+    const uint64_t sgn = neg ? 0x8000000000000000ull : 0ull;
+    z = sa == 0 ? sgn : (dbits(fixed_to_double(sa)) | sgn);
+  } else {
+    const uint64_t cx = mulhi(V, p) << 1;
+    z = cx == 0 ? 0x3ff0000000000000ull : dbits(fixed_to_double((uint64_t)0 - cx));
+  }
+  *sine = SIN == ((q & 1u) == 0);
+  const uint64_t flip = (uint64_t)((*sine ? q : q + 1u) & 2u) << 62;
+  return from_bits(finite ? (z ^ flip) : 0x7ff8000000000000ull);
+}
+
 // sn = sin(2 pi x), cs = cos(2 pi x)
 __host__ __device__ __forceinline__ void sincos2pi_fx(double x, double* sn, double* cs) {
   using namespace fx;
