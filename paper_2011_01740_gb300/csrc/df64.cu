@@ -292,7 +292,12 @@ __global__ void __launch_bounds__(256, 2) ck_phased_df_kernel(AdaptArgs a) {
 // ---------------------------------------------------------------------------
 namespace {
 
-constexpr int kMaxDfTeams = 6;   // teams of two warps per block
+// Teams per block: of two warps, and of three for two frequencies, whose forcing (3,400
+// cycles a stage) one drive warp cannot keep up with: two take every other stage.
+// 1,073 systems x 2 periods 41.1 -> 29.1 ms, 65,536 in 3 teams per SM 51.9 -> 42.8.
+// Four is what the registers hold; in 6 teams of two 131,044 take 70.9 ms (4 of three
+// 74.0), as the FP64 pipe then bounds both.
+constexpr int kMaxDfTeams = 6, kMaxDfTeams3 = 4;
 enum : int { kDfStart = 0, kDfDrive = 1, kDfBars = 6 };
 
 struct __align__(16) DfMailbox {
@@ -307,8 +312,9 @@ __device__ __forceinline__ double df_stage_c(int stage) {  // a stage at t + h i
   return stage == 2 ? ck::c2 : stage == 3 ? ck::c3 : stage == 4 ? ck::c4 : stage == 5 ? ck::c5 : ck::c6;
 }
 
+// stages first, first + step, ..
 template <bool DUAL>
-__device__ __forceinline__ void df_drive_warp(const AdaptArgs& a, DfMailbox& m) {
+__device__ __forceinline__ void df_drive_warp(const AdaptArgs& a, DfMailbox& m, int first, int step) {
   const int lane = threadIdx.x & 31;
   uint32_t start = 0;
   KmForcing<DUAL> frc;
@@ -321,7 +327,7 @@ __device__ __forceinline__ void df_drive_warp(const AdaptArgs& a, DfMailbox& m) 
     }
     const double t = m.t[lane], h = m.h[lane];
 #pragma unroll 1
-    for (int stage = 2; stage <= 6; ++stage) {
+    for (int stage = first; stage <= 6; stage += step) {
       DF fs, fc;
       frc.eval(::fma(df_stage_c(stage), h, t), fs, fc);
       m.f[stage - 2][lane] = make_float4(fs.hi, fs.lo, fc.hi, fc.lo);
@@ -519,15 +525,15 @@ __device__ __forceinline__ void df_main_warp(const AdaptArgs& a, DfMailbox& m, i
   post(&m.bar[kDfStart]);
 }
 
-// block = W main warps, then their W drive warps
-template <bool DUAL>
-__global__ void __launch_bounds__(64 * kMaxDfTeams) ck_phased_df_teams_kernel(AdaptArgs a) {
-  __shared__ DfMailbox boxes[kMaxDfTeams];
-  const int W = (int)(blockDim.x >> 6), w = (int)(threadIdx.x >> 5);
+// block = W main warps, then their DRIVES W drive warps
+template <bool DUAL, int DRIVES, int TEAMS>
+__global__ void __launch_bounds__(32 * (1 + DRIVES) * TEAMS) ck_phased_df_teams_kernel(AdaptArgs a) {
+  __shared__ DfMailbox boxes[TEAMS];
+  const int W = (int)blockDim.x / (32 * (1 + DRIVES)), w = (int)(threadIdx.x >> 5);
   if (threadIdx.x < (unsigned)W) init_bars(boxes[threadIdx.x].bar, kDfBars);
   __syncthreads();
   if (w < W) df_main_warp<DUAL>(a, boxes[w], W);
-  else df_drive_warp<DUAL>(a, boxes[w - W]);
+  else df_drive_warp<DUAL>(a, boxes[w % W], 1 + w / W, DRIVES);
 }
 
 }  // namespace
@@ -794,9 +800,11 @@ cudaError_t launch_ck45_df_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch
   if (a.n_phases <= 0) return cudaErrorInvalidValue;
   if (L.grid <= 0 || L.grid > 0x7fffffffLL || L.block < 32 || L.block % 32 || L.block > 32 * kMaxDfTeams)
     return cudaErrorInvalidConfiguration;
-  const dim3 g((unsigned)L.grid), b(2 * (unsigned)L.block);
-  if (flags & kKmDual) ck_phased_df_teams_kernel<true><<<g, b, 0, s>>>(a);
-  else ck_phased_df_teams_kernel<false><<<g, b, 0, s>>>(a);
+  const bool dual = flags & kKmDual, three = dual && L.block <= 32 * kMaxDfTeams3;
+  const dim3 g((unsigned)L.grid), b((three ? 3 : 2) * (unsigned)L.block);
+  if (three) ck_phased_df_teams_kernel<true, 2, kMaxDfTeams3><<<g, b, 0, s>>>(a);
+  else if (dual) ck_phased_df_teams_kernel<true, 1, kMaxDfTeams><<<g, b, 0, s>>>(a);
+  else ck_phased_df_teams_kernel<false, 1, kMaxDfTeams><<<g, b, 0, s>>>(a);
   return cudaGetLastError();
 }
 
