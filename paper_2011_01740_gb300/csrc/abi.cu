@@ -57,6 +57,7 @@ struct ens_ctx {
   unsigned* hist = nullptr;     // histogram scratch of the claim-order sort
   Scratch* scratch = nullptr;
   ens_launch launch{};
+  bool launch_set = false;   // by the caller or the tuner; else it follows the parameters
   // CUDA graph of one solve
   cudaGraphExec_t gexec = nullptr;
   cudaStream_t graph_stream = nullptr;
@@ -100,19 +101,25 @@ ens_status cuda_fail(ens_ctx* c, cudaError_t e, const char* what) {
 // to 6 periods or 16 time units); all shapes give the same results.
 //   Up to one warp per SM sub-partition (128 systems per SM) every system
 //   starts at once, so an order only costs its pilot, and blocks of one warp
-//   put each warp on a sub-partition of its own: 1,073 bubbles 45.4 against
-//   51.7 (160 x 1, longest first), 15,000 45.6 / 52.7, 4,608 frequencies 141.7 /
-//   147.7, split precision 16,384 14.4 / 17.4.
-//   Above that the longest systems bound the run until there are enough
-//   others.  FP64 Keller-Miksis phases want 5 teams of three warps per SM (kernel
-//   alone, 131,044 x 4: 110.6, 6 plain warps 126.3; 65,536 x 2: 39.7 / 49.0), then 8
-//   plain warps (200,000 x 2: 78.5, 5 teams 80.3), then 12 (262,144 x 2: 101.9 /
+//   put each warp on a sub-partition of its own: FP64 without a team kernel,
+//   split precision 16,384 14.4 against 17.4 (160 x 1, longest first).
+//   FP64 Keller-Miksis phases with teams: a relay holds a warp of systems and two
+//   fit on an SM, so up to there (64 systems per SM) all start at once (5,120: 21.3,
+//   with an order 22.7); above, one relay per SM that claims the longest first
+//   (19,200: 22.8, all at once in teams 35.0), then two (25,600: 25.1, one 27.6;
+//   51,200: 31.5, 3 teams 38.1), then 3 teams (65,536: 38.7, two relays 39.7), 4
+//   (90,000, kernel alone: 40.7, 3 teams 49.6), 5 (131,044 x 2: 52.4, 4 teams 59.0;
+//   x 4: 110.6, 6 plain warps 126.3), then 8 plain
+//   warps (200,000 x 2: 78.5, 5 teams 80.3), then 12 (262,144 x 2: 97.0, 5 teams
 //   105.1; 524,288: 199 / 209); other FP64 phases 5 warps (65,536: 57.6, 6 warps
-//   58.9), then 6 (131,044: 207 / 221 at 5), then 12.  Split precision: 8 (131,044: 19.1 / 20.4), 12
-//   (262,144: 23.6 / 38.2), 16 (524,288: 37.9 / 74.9), 24 from there.
-//   Double-float phases 3 teams of two warps per SM (kernel alone, 65,536 x 4:
-//   72.3, 4 teams 73.9), then 6 (131,044 x 2: 41.9, 4 teams 54.9), then 12 plain
-//   warps (262,144 x 2: 60.8, 8 warps 71.1), then 16 (524,288 x 2: 111.6, 12 120.9).
+//   58.9), then 6 (131,044: 207 / 221 at 5), then 12.  Split precision, kernels
+//   alone: 4 (65,536 x 4: 14.2, 8 warps 16.0), then 8 (131,044: 16.2, 4 warps 20.5), 12
+//   (262,144: 19.5 / 23.1 at 8), 16 (524,288: 37.9 / 74.9 at 5), 24 from there.
+//   Double-float phases, kernels alone: teams on 2 of the sub-partitions (32,768 x 4:
+//   54.0, 3 teams 61.0), 3 (65,536: 61.9, 2 teams 80.6), 4 (90,000: 65.8, 3 teams 84.1),
+//   6 (131,044: 81.8, 4 teams 95.2), then 12 plain warps (262,144 x 2: 60.8, 8 warps
+//   71.1), then 16 (524,288 x 2: 111.6, 12 120.9).  Two frequencies leave the plain
+//   launch earlier, as four teams of three warps do not fit (19,200 x 2: 40.8 / 29.2).
 //   Valves take about the same number of steps each, and neighbours take them
 //   alike, which claiming by cost breaks up: plain launches of 1 warp a block
 //   (1,000: 21.5 / 25.4; 32,768: 25.8 / 37.2; 65,536: 46.4 / 60.7; 262,144: 168 /
@@ -131,7 +138,8 @@ ens_launch default_launch(const ens_ctx* c) {
     if (c->tol.prec == ENS_FP32X2) L.block = 256;
     return L;
   }
-  if (c->n <= (int64_t)c->sm_count * 128) {
+  const bool teams = has_teams(c), dual_df = c->tol.prec == ENS_FP32X2 && (c->km_flags & kKmDual);
+  if (c->n <= (int64_t)c->sm_count * (teams || dual_df ? 64 : 128)) {
     if (c->tol.prec == ENS_FP32X2) L.block = 64;  // 16,384 x 2: 33.0, one warp a block 35.7
     return L;
   }
@@ -139,14 +147,19 @@ ens_launch default_launch(const ens_ctx* c) {
   L.blocks_per_sm = 1;
   L.cost_order = 1;
   if (c->tol.prec == ENS_FP32_COMP) {
-    L.block = per_sm >= 1300 && per_sm < 2600 ? 128 : 256;
+    L.block = per_sm < 700 || (per_sm >= 1300 && per_sm < 2600) ? 128 : 256;
     L.blocks_per_sm = per_sm < 1300 ? 1 : per_sm < 2600 ? 3 : per_sm < 5200 ? 2 : 3;
   } else if (c->tol.prec == ENS_FP32X2) {
-    L.block = per_sm < 640 ? 96 : per_sm < 1300 ? 192 : per_sm < 2600 ? 128 : 256;
+    L.block = per_sm < 320 ? 64 : per_sm < 440 ? 96 : per_sm < 710 ? 128 : per_sm < 1300 ? 192 : per_sm < 2600 ? 128 : 256;
     L.blocks_per_sm = per_sm < 1300 ? 1 : per_sm < 2600 ? 3 : 2;
+  } else if (teams && per_sm < 410) {
+    L.block = 32;
+    L.blocks_per_sm = per_sm < 145 ? 1 : 2;
+  } else if (teams && per_sm < 1300) {
+    L.block = per_sm < 480 ? 96 : per_sm < 600 ? 128 : 160;
   } else if (per_sm < 1300) {
-    L.block = per_sm < 640 || has_teams(c) ? 160 : 192;
-  } else if (per_sm < 1700 && has_teams(c)) {
+    L.block = per_sm < 640 ? 160 : 192;
+  } else if (per_sm < 1700 && teams) {
     L.block = 256;
   } else {
     L.block = 128;
@@ -236,12 +249,11 @@ bool teams_fit(const ens_ctx* c, AdaptLaunch L) {
   return has_teams(c) && L.spt == 1 && L.block <= 160 && L.grid * (L.block / 32) <= 5 * (int64_t)c->sm_count;
 }
 
-// Whether they run in relays (rkck45_relay.cu): blocks of one warp of systems, up to
-// two per SM, which is what the registers hold.  Up to there the longest system
-// bounds the run, and its trial takes two thirds of the teams' time (1 system 30.3 /
-// 19.5 ms, 9,700 x 2 periods 32.6 / 21.9).
+// Of those, up to two warps of systems per SM run in relays (rkck45_relay.cu), which
+// is what the registers hold: the longest system bounds the run, and its trial takes
+// two thirds of the teams' time (1 system 30.3 / 19.5 ms, 9,700 x 2 periods 32.6 / 21.9).
 bool relay_fits(const ens_ctx* c, AdaptLaunch L) {
-  return has_teams(c) && L.spt == 1 && L.block == 32 && L.grid <= 2 * (int64_t)c->sm_count;
+  return teams_fit(c, L) && L.grid * (L.block / 32) <= 2 * (int64_t)c->sm_count;
 }
 
 // The same for double-float phases, in teams of two (df64.cu): up to 6 per SM
@@ -259,7 +271,7 @@ cudaError_t launch_adaptive(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L,
     return df_teams_fit(c, L) ? launch_ck45_df_teams(c->km_flags, a, L, s) : launch_ck45_df(c->km_flags, a, L, s);
   }
   if (L.spt == 2) return launch_ck45_spt2(c->sys, c->km_flags, a, L, s);
-  if (relay_fits(c, L)) return launch_ck45_relay(c->km_flags, a, L, s);
+  if (relay_fits(c, L)) return launch_ck45_relay(c->km_flags, a, AdaptLaunch{L.grid * (L.block / 32), 32}, s);
   if (teams_fit(c, L)) return launch_ck45_teams(c->km_flags, a, L, s);
   return launch_ck45(c->sys, c->km_flags, a, L, s);
 }
@@ -658,7 +670,10 @@ ens_status ens_set_inputs(ens_ctx* c, const double* params, const double* y0, vo
     const unsigned was = c->km_flags;
     ens_status st = detect_flags(c);
     if (st != ENS_OK) return st;
-    if (was != c->km_flags) c->graph_valid = false;
+    if (was != c->km_flags) {
+      c->graph_valid = false;
+      if (!c->launch_set) c->launch = default_launch(c);
+    }
   }
   return ENS_OK;
 }
@@ -679,6 +694,7 @@ ens_status ens_set_launch(ens_ctx* c, const ens_launch* cfg) {
     return ENS_ENOTSUP;
   }
   c->launch = L;
+  c->launch_set = cfg != nullptr;
   c->graph_valid = false;
   return ENS_OK;
 }
@@ -803,6 +819,7 @@ ens_status ens_autotune(ens_ctx* c, void* stream, ens_launch* best) {
     if (it != g_tune_cache.end()) {
       const bool graph = c->launch.use_graph;
       c->launch = it->second.first;
+      c->launch_set = true;
       c->launch.use_graph = graph;
       c->tune_rows = it->second.second;
       c->graph_valid = false;
@@ -899,6 +916,10 @@ ens_status ens_autotune(ens_ctx* c, void* stream, ens_launch* best) {
     // warps per SM -> (block, blocks per SM)
     const int shapes[][3] = {{3, 96, 1},  {4, 128, 1},  {5, 160, 1},  {6, 192, 1},  {7, 224, 1},
                              {8, 256, 1}, {12, 192, 2}, {16, 256, 2}, {24, 256, 3}};
+    // relays, where not every system starts at once
+    if (has_teams(c) && c->n > 64 * (int64_t)c->sm_count)
+      for (const int bps : {1, 2})
+        if (st == ENS_OK) st = consider(mk(ENS_LAUNCH_PERSISTENT, 32, bps, 1, 1));
     int best_w = 0;
     for (const auto& sh : shapes) {
       if (st != ENS_OK) break;
@@ -938,6 +959,7 @@ ens_status ens_autotune(ens_ctx* c, void* stream, ens_launch* best) {
   if (st != ENS_OK) return st;
   best_L.use_graph = c->launch.use_graph;
   c->launch = best_L;
+  c->launch_set = true;
   c->graph_valid = false;
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);

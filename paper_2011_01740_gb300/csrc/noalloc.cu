@@ -184,11 +184,13 @@ extern "C" ens_status ens_solve_noalloc(ens_system sys, int64_t n, const double*
   const int64_t need = (n + 127) / 128;
   if (grid > need) grid = need;
   if (grid < 1) grid = 1;
-  // Keller-Miksis with the exponent 21/5: relays up to two warps of systems per SM (1,073
-  // x 2 periods 33 -> 21 ms), else teams, whose range ends at five
+  // Keller-Miksis with the exponent 21/5: relays, two per SM at most (1,073 x 2 periods
+  // 33 -> 21 ms; 40,000 x 2 38 with two relays per SM in any order, 26 longest first, 41 in
+  // 4 teams), then teams, whose range ends at five
   const bool teams = sys == ENS_SYS_KELLER_MIKSIS && !(flags & kKmGeneralExponent);
-  const bool relay = teams && n <= 64 * (int64_t)sms;
-  if ((relay   ? launch_ck45_relay(flags, a, AdaptLaunch{(n + 31) / 32, 32}, s)
+  const bool relay = teams && n < (cost_order ? 410 : 260) * (int64_t)sms;
+  const int64_t relays = (n + 31) / 32 < 2 * (int64_t)sms ? (n + 31) / 32 : 2 * (int64_t)sms;
+  if ((relay   ? launch_ck45_relay(flags, a, AdaptLaunch{relays, 32}, s)
        : teams ? launch_ck45_teams(flags, a, AdaptLaunch{grid, 128}, s)
                : launch_ck45(sys, flags, a, AdaptLaunch{grid, 128}, s)) != cudaSuccess)
     return fail(ENS_ECUDA, "ens_solve_noalloc: launch failed");

@@ -27,11 +27,14 @@ def _same(ctx):
     return default
 
 
-@pytest.mark.parametrize("prec,n", [(ens.ENS_FP64, 1), (ens.ENS_FP64, 128 * SMS), (ens.ENS_FP64, 128 * SMS + 1),
-                                    (ens.ENS_FP64, 640 * SMS), (ens.ENS_FP64, 1300 * SMS),
+@pytest.mark.parametrize("prec,n", [(ens.ENS_FP64, 1), (ens.ENS_FP64, 64 * SMS), (ens.ENS_FP64, 64 * SMS + 1),
+                                    (ens.ENS_FP64, 145 * SMS), (ens.ENS_FP64, 410 * SMS), (ens.ENS_FP64, 480 * SMS),
+                                    (ens.ENS_FP64, 600 * SMS), (ens.ENS_FP64, 1300 * SMS),
+                                    (ens.ENS_FP32_COMP, 128 * SMS), (ens.ENS_FP32_COMP, 700 * SMS),
                                     (ens.ENS_FP32_COMP, 128 * SMS + 1), (ens.ENS_FP32_COMP, 1300 * SMS),
                                     (ens.ENS_FP32_COMP, 2600 * SMS), (ens.ENS_FP32X2, 33),
-                                    (ens.ENS_FP32X2, 640 * SMS + 1)])
+                                    (ens.ENS_FP32X2, 64 * SMS + 1), (ens.ENS_FP32X2, 320 * SMS),
+                                    (ens.ENS_FP32X2, 440 * SMS), (ens.ENS_FP32X2, 710 * SMS)])
 @pytest.mark.parametrize("dual", [False, True])
 def test_keller_miksis_default_launch(prec, n, dual):
     """One short period; the dual-frequency runs also take the split-precision
@@ -39,12 +42,15 @@ def test_keller_miksis_default_launch(prec, n, dual):
     km = (W.km_dual if dual else W.km)(1, n, n_phases=1, pa_max=0.6e5, f_min=2e5)
     ph = km["phys"]
     ph["pA1"][:] = np.linspace(0.2e5, 0.6e5, n)
+    if dual:
+        ph["pA2"][:] = 0.5 * ph["pA1"]
     C = ens.ens_km_coefficients(*[ph[k] for k in ("pA1", "f1", "pA2", "f2", "theta", "RE")], km["liquid"])
     tol = ens.make_tol(rtol=1e-7, atol=1e-7, n_phases=1, prec=prec)
     ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS, n, C, km["y0"], (0.0, 1.0), ens.ENS_RKCK45, tol)
     try:
         default = _same(ctx)
-        assert (default["mode"] == ens.ENS_LAUNCH_PLAIN) == (n <= 128 * SMS)
+        once = 64 if prec == ens.ENS_FP64 or (dual and prec == ens.ENS_FP32X2) else 128   # all start at once
+        assert (default["mode"] == ens.ENS_LAUNCH_PLAIN) == (n <= once * SMS)
     finally:
         ens.ens_destroy(ctx)
 
@@ -58,5 +64,29 @@ def test_valve_default_launch(prec, n):
     ctx = ens.ens_create(ens.ENS_SYS_RELIEF_VALVE, n, w["params"], w["y0"], (0.0, 1.0), ens.ENS_RKCK45, tol)
     try:
         assert _same(ctx)["mode"] == ens.ENS_LAUNCH_PLAIN
+    finally:
+        ens.ens_destroy(ctx)
+
+
+def test_default_launch_follows_the_parameters():
+    """A context that only ever had the default changes it with the exponent that
+    decides on the team kernels; one whose caller chose keeps the choice."""
+    n = 64 * SMS + 1
+    km = W.km(1, n, n_phases=1, pa_max=0.6e5)
+    ph = km["phys"]
+    C = ens.ens_km_coefficients(*[ph[k] for k in ("pA1", "f1", "pA2", "f2", "theta", "RE")], km["liquid"])
+    other = C.copy()
+    other[10] = 4.0
+    ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS, n, C, km["y0"], (0.0, 1.0), ens.ENS_RKCK45, ens.make_tol(n_phases=1))
+    try:
+        mode = lambda: ens.ens_get_launch(ctx).mode
+        assert mode() == ens.ENS_LAUNCH_PERSISTENT
+        ens.ens_set_inputs(ctx, other, km["y0"])
+        assert mode() == ens.ENS_LAUNCH_PLAIN
+        ens.ens_set_inputs(ctx, C, km["y0"])
+        assert mode() == ens.ENS_LAUNCH_PERSISTENT
+        ens.ens_set_launch(ctx, ens.make_launch(mode=ens.ENS_LAUNCH_PERSISTENT, block=96, blocks_per_sm=1))
+        ens.ens_set_inputs(ctx, other, km["y0"])
+        assert ens.ens_get_launch(ctx).block == 96
     finally:
         ens.ens_destroy(ctx)

@@ -27,7 +27,10 @@ def _compare(n, launch, solver=ens.ENS_RKCK45, dual=False, t0=0.0, **tol):
     km = (W.km_dual if dual else W.km)(1, n, pa_max=1e5)
     km["phys"]["pA1"][:] = np.random.default_rng(n).uniform(0.0, 1.2e5, n)
     ph = km["phys"]
+    if dual:
+        ph["pA2"][:] = 0.5 * ph["pA1"]
     C = ens.ens_km_coefficients(*[ph[k] for k in ("pA1", "f1", "pA2", "f2", "theta", "RE")], km["liquid"])
+    assert np.any(C[6]) == dual
     t = ens.make_tol(**{**dict(rtol=1e-8, atol=1e-8, n_phases=3), **tol})
     ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS, n, C, km["y0"], (t0, t0 + 1.0), solver, t)
     try:
