@@ -344,10 +344,10 @@ AdaptLaunch adapt_launch(const ens_ctx* c, const ens_launch& L) {
 // of the horizon) of every system in plain mode, then the systems sorted by
 // decreasing pilot step count into c->order.  The pilot only ranks the
 // systems (the claim order never changes what a system computes), so it runs at
-// a tolerance of at least kPilotTol, a quarter of the steps of a 1e-10 pilot,
+// a tolerance of at least kPilotTol, a tenth of the steps of a 1e-10 pilot,
 // and Keller-Miksis phases are ranked in split precision: a trial of the
 // longest system, which bounds the pilot, takes 2.9 us there against 10.4 us
-// in FP64 (131,044 systems: pilot and sort 14 ms in FP64, 4 ms now).
+// in FP64 (131,044 systems: pilot and sort 1.6 ms, at 1e-7 in FP64 14).
 // kPilotTrials bounds a system whose float pilot would be held up by rounding; it
 // ranks with the longest.
 ens_status enqueue_order(ens_ctx* c, const AdaptArgs& a, cudaStream_t s) {
