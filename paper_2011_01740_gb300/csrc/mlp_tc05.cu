@@ -116,8 +116,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) mlp_forward_tc05_kernel(TcArgs 
       for (int j = 0; j < 4; ++j) {
         const float4 w = *reinterpret_cast<const float4*>(sW1 + 2 * (kc * 8 + 2 * j));
         const float2 b = b1[kc * 4 + j];
-        h[2 * j] = gelu(fmaf(w.y, x1, fmaf(w.x, x0, b.x)));
-        h[2 * j + 1] = gelu(fmaf(w.w, x1, fmaf(w.z, x0, b.y)));
+        h[2 * j] = fmaf(w.y, x1, fmaf(w.x, x0, b.x));
+        h[2 * j + 1] = fmaf(w.w, x1, fmaf(w.z, x0, b.y));
+        gelu2(h[2 * j], h[2 * j + 1]);
       }
       store_bf16x8(tile, row, kc * 8, h);
     }
@@ -142,10 +143,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) mlp_forward_tc05_kernel(TcArgs 
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
           const float4 b = *reinterpret_cast<const float4*>(bl + c * 32 + 4 * q);
-          v[4 * q] = gelu(v[4 * q] + b.x);
-          v[4 * q + 1] = gelu(v[4 * q + 1] + b.y);
-          v[4 * q + 2] = gelu(v[4 * q + 2] + b.z);
-          v[4 * q + 3] = gelu(v[4 * q + 3] + b.w);
+          bias_gelu2(v[4 * q], v[4 * q + 1], b.x, b.y);
+          bias_gelu2(v[4 * q + 2], v[4 * q + 3], b.z, b.w);
         }
         if (l < 2) {
 #pragma unroll

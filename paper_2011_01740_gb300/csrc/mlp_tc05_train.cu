@@ -208,10 +208,12 @@ __global__ void __launch_bounds__(kT, 1) mlp_step_tc05_kernel(TrainTcArgs a) {
           const uint32_t ww[4] = {w.x, w.y, w.z, w.w};
           const float b[4] = {ba.x, ba.y, bb.x, bb.y};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float z = fmaf(bf16_hi(ww[j]), x1, fmaf(bf16_lo(ww[j]), x0, b[j]));
-            gelu_and_grad(z, h[4 * u + j], gq[4 * u + j]);
-            if (!live) h[4 * u + j] = 0.f;
+          for (int j = 0; j < 4; j += 2) {
+            const int c = 4 * u + j;
+            gelu_and_grad2(df::f2(fmaf(bf16_hi(ww[j]), x1, fmaf(bf16_lo(ww[j]), x0, b[j])),
+                                  fmaf(bf16_hi(ww[j + 1]), x1, fmaf(bf16_lo(ww[j + 1]), x0, b[j + 1]))),
+                           h[c], h[c + 1], gq[c], gq[c + 1]);
+            if (!live) h[c] = h[c + 1] = 0.f;
           }
         }
         store_bf16x8(ring(), s, c0 + 8 * q, h);
@@ -228,12 +230,9 @@ __global__ void __launch_bounds__(kT, 1) mlp_step_tc05_kernel(TrainTcArgs a) {
       wait();
       tmem_ld32(mine + kAcc, v);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        v[2 * j] += b[j].x;
-        v[2 * j + 1] += b[j].y;
-      }
-#pragma unroll
-      for (int j = 0; j < 32; ++j) gelu_and_grad(v[j], v[j], g[j]);
+      for (int j = 0; j < 16; ++j)
+        gelu_and_grad2(df::add_f(df::f2(v[2 * j], v[2 * j + 1]), df::f2(b[j].x, b[j].y)), v[2 * j], v[2 * j + 1],
+                       g[2 * j], g[2 * j + 1]);
       if (l < 4) {
         if (!live) {
 #pragma unroll
