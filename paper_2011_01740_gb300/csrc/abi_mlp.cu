@@ -119,6 +119,8 @@ void free_batch(ens_mlp* m) {
   m->cap = 0;
 }
 
+__host__ __device__ constexpr df::DF pair_of(double x) { return df::DF{(float)x, (float)(x - (double)(float)x)}; }
+
 // the shuffle buffers of a run over more samples than this are given back after it
 constexpr int64_t kKeepShuffle = 1 << 24;
 
@@ -274,11 +276,53 @@ ens_status set_smem_attrs(ens_mlp* m) {
 // screening-pipeline helpers
 // ---------------------------------------------------------------------------
 
+// A feature 2 (log v - l0) / (l1 - l0) - 1, rounded to float.  Logarithm and division
+// in FP64 held the FP64 pipe for 75 instructions a point (4.2 M points: 665 us);
+// double-float pairs (df.cuh) on the FP32 pipes give the value to within 2^-42 of
+// its terms, and the float that it rounds to is the FP64 formula's unless a rounding
+// boundary lies within twice that.  Then, and for v that is not positive and
+// normal, the FP64 formula decides.
+struct LogFeature {
+  double l0, l1;
+  df::DF l0p, scale;   // l0 and 2 / (l1 - l0) as pairs
+  float margin, per_log;
+  __device__ __forceinline__ LogFeature(double a, double b) : l0(a), l1(b) {
+    const double s = 2.0 / (b - a);
+    l0p = df::from_double(a);
+    scale = df::from_double(s);
+    per_log = 0x1p-41f * (float)s;
+    margin = 0x1p-41f * (2.0f + (float)(s * fabs(a)));
+  }
+  __device__ __forceinline__ float operator()(double v) const {
+    using namespace df;
+    const long long bits = __double_as_longlong(v);
+    const int ef = (int)(bits >> 52);   // with the sign: positive and normal in [1, 0x7fe]
+    // v = m 2^e, m in [0.7, 1.42): log v = e ln 2 + 2 atanh z, z = (m - 1) / (m + 1)
+    const bool high = (bits & 0x000fffffffffffffLL) >= 0x6a09e667f3bcdLL;   // m >= sqrt 2
+    const int e = ef - (high ? 1022 : 1023);
+    const DF m = from_double(__longlong_as_double((bits & 0x000fffffffffffffLL) | ((long long)(high ? 1022 : 1023) << 52)));
+    const DF z = mul(add(m, -1.0f), rcp(add(m, 1.0f)));
+    const DF w = mul(z, z);
+    // 1 + w/3 + w^2/5 + ..: w < 0.0295, the terms from w^4 on in single precision, the rest below 2^-50
+    const float t = fmaf(w.hi, fmaf(w.hi, fmaf(w.hi, fmaf(w.hi, 1.0f / 17, 1.0f / 15), 1.0f / 13), 1.0f / 11), 1.0f / 9);
+    DF s = add(mul(w, t), pair_of(1.0 / 7));
+    s = add(mul(w, s), pair_of(1.0 / 5));
+    s = add(mul(w, s), pair_of(1.0 / 3));
+    s = add(mul(w, s), 1.0f);
+    const DF l = add(mul(pair_of(0.693147180559945309417232), (float)e), mul(DF{2.0f * z.hi, 2.0f * z.lo}, s));
+    const DF x = add(mul(sub(l, l0p), scale), -1.0f);
+    const float d = fmaf(per_log, fabsf(l.hi), margin);
+    const bool safe = ef >= 1 && ef <= 0x7fe && add_f(x.hi, add_f(x.lo, d)) == x.hi && add_f(x.hi, sub_f(x.lo, d)) == x.hi;
+    return safe ? x.hi : (float)(2.0 * (log(v) - l0) / (l1 - l0) - 1.0);
+  }
+};
+
 __global__ void km_features_kernel(int64_t n, const double* pA, const double* f, double la0, double la1,
                                    double lf0, double lf1, float* x) {
+  const LogFeature A(la0, la1), F(lf0, lf1);
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    x[2 * i] = (float)(2.0 * (log(pA[i]) - la0) / (la1 - la0) - 1.0);
-    x[2 * i + 1] = (float)(2.0 * (log(f[i]) - lf0) / (lf1 - lf0) - 1.0);
+    x[2 * i] = A(pA[i]);
+    x[2 * i + 1] = F(f[i]);
   }
 }
 
