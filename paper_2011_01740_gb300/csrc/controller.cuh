@@ -68,8 +68,8 @@ __device__ __forceinline__ int64_t claim(const AdaptArgs& a, bool first, int lan
 // longest systems), the others the next ones; later claims continue from rank
 // gridDim.x * lanes in order (claim_next_after_ranked).  The claim order
 // never changes what a system computes.
-__device__ __forceinline__ int64_t claim_first_by_subpartition(const AdaptArgs& a, int W) {
-  const int w = (int)(threadIdx.x >> 5), lane = (int)(threadIdx.x & 31);
+__device__ __forceinline__ int64_t claim_first_by_subpartition(const AdaptArgs& a, int W, int w) {
+  const int lane = (int)(threadIdx.x & 31);
   int u_total = 0, u_before = 0;
   for (int x = 0; x < W; ++x) {
     const bool own = ((W - (x & 3) + 3) >> 2) == 1;  // the only warp of block x's sub-partition

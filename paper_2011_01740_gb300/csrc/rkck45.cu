@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(256) ck_phased_kernel(AdaptArgs a) {
   constexpr int D = Sys::kDim;
   const double tau_end = a.t0 + a.phase_len;
   const uint64_t deadline = global_ns() + a.timeout_ns;
-  int64_t i = a.first_by_subpartition ? claim_first_by_subpartition(a, (int)(blockDim.x >> 5))
+  int64_t i = a.first_by_subpartition ? claim_first_by_subpartition(a, (int)(blockDim.x >> 5), (int)(threadIdx.x >> 5))
                                       : claim(a, true, (int)blockDim.x, (int)threadIdx.x);
   bool timed_out = false;
   Sys s;

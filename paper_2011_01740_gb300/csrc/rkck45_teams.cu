@@ -32,11 +32,12 @@
 // of an SM run in step, 151 ms on 131,044 x 4 when they do not: instruction cache);
 // the power spelled out a stage earlier in the one-warp kernel (45.3 -> 50.6 ms).
 //
-// Messages go through a mailbox in shared memory, each kind on an mbarrier of its
-// own: the sender's lanes write, one lane arrives; the receiver waits for the
-// phase.  A slot is used again only after its reply has been received, and the
-// drive warp starts a trial only when the main warp does, so no barrier is ever
-// more than one phase ahead of its receiver.  Waits are bounded; when one of the
+// Messages go through a mailbox in shared memory, on mbarriers with one phase per
+// trial: the sender's lanes write, one lane arrives; the receiver waits for the
+// phase.  A stage's power and drive arrive on one barrier (a wait costs some 60 cycles:
+// 131,044 x 3 periods 81.8 -> 81.1 ms).  The main warp has received everything of a
+// trial before it starts the next, so no barrier is ever more than one phase ahead of
+// its receiver.  Waits are bounded; when one of the
 // main warp's expires, its systems and all it still claims are retired with
 // ENS_SYS_TIMEOUT, and a helper whose wait expires leaves.
 #include "common.cuh"
@@ -51,11 +52,11 @@ namespace {
 constexpr int kMaxTeams = 5;             // teams of three warps per block
 
 // barriers of a team's mailbox
-enum : int { kReq = 0, kRsp = 2, kCtlReq = 4, kCtlRsp = 5, kStart = 6, kDrive = 7, kBars = 12 };
+enum : int { kReq = 0, kAll = 6, kCtlReq = 12, kCtlRsp = 13, kStart = 14, kBars = 15 };
 
 struct __align__(16) Mailbox {
-  double x[2][32];             // power request: y1 of a stage
-  double g[2][32];             // its reply
+  double x[6][32];             // power request: y1 of a stage
+  double g[6][32];             // its reply
   double t[32], h[32];         // trial start: its time and length,
   long long sys[32];           //              the lane's system
   double fs[5][32], fc[5][32]; // drives of stages 2..6
@@ -73,6 +74,11 @@ __device__ __forceinline__ double stage_c(int stage) {
   return stage == 2 ? ck::c2 : stage == 3 ? ck::c3 : stage == 4 ? ck::c4 : stage == 5 ? ck::c5 : ck::c6;
 }
 
+// the next phase of a barrier that has one per trial
+__device__ __forceinline__ bool all_await(Mailbox& m, int bar, uint32_t trial) {
+  return __all_sync(0xffffffffu, await(&m.bar[bar], trial));
+}
+
 // Both helpers' loops over the stages stay rolled: unrolled (50 KB) they thrash the
 // instruction cache as soon as the teams of an SM run out of step.
 
@@ -80,18 +86,16 @@ __device__ __forceinline__ double stage_c(int stage) {
 template <class Sys>
 __device__ __forceinline__ void power_warp(const AdaptArgs& a, Mailbox& m) {
   const int lane = threadIdx.x & 31;
-  uint32_t r0 = 0, r1 = 0, creq = 0;
   const Sys s{};
-  for (;;) {
+  for (uint32_t trial = 0;; ++trial) {
 #pragma unroll 1
     for (int k = 0; k < 6; ++k) {
-      const int slot = k & 1;
-      if (!__all_sync(0xffffffffu, await(&m.bar[kReq + slot], slot ? r1 : r0))) return;
+      if (!all_await(m, kReq + k, trial)) return;
       if (k == 0 && !m.run) return;
-      m.g[slot][lane] = s.early_power(m.x[slot][lane]);
-      post(&m.bar[kRsp + slot]);
+      m.g[k][lane] = s.early_power(m.x[k][lane]);
+      post(&m.bar[kAll + k]);
     }
-    if (!__all_sync(0xffffffffu, await(&m.bar[kCtlReq], creq))) return;
+    if (!all_await(m, kCtlReq, trial)) return;
     const double y[2] = {m.v[0][lane], m.v[1][lane]}, y5[2] = {m.v[2][lane], m.v[3][lane]},
                  err[2] = {m.v[4][lane], m.v[5][lane]};
     const double E = err_norm<2>(y, y5, err, a.rtol, a.atol);
@@ -105,11 +109,10 @@ __device__ __forceinline__ void power_warp(const AdaptArgs& a, Mailbox& m) {
 template <class Sys, int PAIR>
 __device__ __forceinline__ void drive_warp(const AdaptArgs& a, Mailbox& m) {
   const int lane = threadIdx.x & 31;
-  uint32_t start = 0;
   Sys s;
   long long cur = -1;
-  for (;;) {
-    if (!__all_sync(0xffffffffu, await(&m.bar[kStart], start)) || !m.run) return;
+  for (uint32_t trial = 0;; ++trial) {
+    if (!all_await(m, kStart, trial) || !m.run) return;
     if (m.sys[lane] != cur) {
       cur = m.sys[lane];
       s.load(a.params, a.n, cur);
@@ -120,17 +123,17 @@ __device__ __forceinline__ void drive_warp(const AdaptArgs& a, Mailbox& m) {
       const typename Sys::Drive d = s.drive(fma(stage_c<PAIR>(stage), h, t));
       m.fs[stage - 2][lane] = d.fs;
       m.fc[stage - 2][lane] = d.fc;
-      post(&m.bar[kDrive + stage - 2]);
+      post(&m.bar[kAll + stage - 2]);
     }
   }
 }
 
 template <class Sys, int PAIR>
-__device__ __forceinline__ void main_warp(const AdaptArgs& a, Mailbox& m, int W) {
+__device__ __forceinline__ void main_warp(const AdaptArgs& a, Mailbox& m, int W, int w) {
   const int lane = threadIdx.x & 31, lanes = 32 * W;
   const double tau_end = a.t0 + a.phase_len;
   const uint64_t deadline = global_ns() + a.timeout_ns;
-  uint32_t rsp[2] = {0, 0}, crsp = 0, drv = 0, iter = 0;
+  uint32_t trial = 0, iter = 0;
   bool timed_out = false, dead = false;
   Sys s;
   typename Sys::Drive d0, dn;  // drive at the phase start, at the end of the trial
@@ -187,8 +190,8 @@ __device__ __forceinline__ void main_warp(const AdaptArgs& a, Mailbox& m, int W)
     return a.first_by_subpartition ? claim_next_after_ranked(a, lanes) : claim(a, false, 0, 0);
   };
 
-  int64_t i = a.first_by_subpartition ? claim_first_by_subpartition(a, W)
-                                      : claim(a, true, lanes, (int)threadIdx.x);
+  int64_t i = a.first_by_subpartition ? claim_first_by_subpartition(a, W, w)
+                                      : claim(a, true, lanes, 32 * w + lane);
   long long shown = i >= 0 ? i : 0;   // a lane without a system computes on system 0 and stores nothing
   start_system(shown);
 
@@ -224,18 +227,15 @@ __device__ __forceinline__ void main_warp(const AdaptArgs& a, Mailbox& m, int W)
     bool ok = true;
     // the rest of a stage's acceleration with its power, requested earlier, and drive
     auto finish_stage = [&](int stage, const typename Sys::Half& p, typename Sys::Drive& d) {
-      const int slot = stage & 1;
-      ok &= await(&m.bar[kRsp + slot], rsp[slot]);
-      const typename Sys::Half2 q = s.accel_more(p);   // the pipe works while g arrives
-      const double N = s.accel_mid(p, q, m.g[slot][lane]);
-      uint32_t phase = drv;   // one phase per trial
-      ok &= await(&m.bar[kDrive + stage - 2], phase);
+      uint32_t phase = trial;   // one phase per trial
+      ok &= await(&m.bar[kAll + stage - 2], phase);
+      const typename Sys::Half2 q = s.accel_more(p);   // the pipe works while they arrive
       d = {m.fs[stage - 2][lane], m.fc[stage - 2][lane]};
-      return s.accel_last(p, q, N, d.fs, d.fc);
+      return s.accel_last(p, q, s.accel_mid(p, q, m.g[stage - 2][lane]), d.fs, d.fc);
     };
-    auto request = [&](int slot, double x) {
-      m.x[slot][lane] = x;
-      post(&m.bar[kReq + slot]);
+    auto request = [&](int stage, double x) {
+      m.x[stage - 2][lane] = x;
+      post(&m.bar[kReq + stage - 2]);
     };
     if constexpr (PAIR == kCashKarp) {
       typename Sys::Drive d;
@@ -245,36 +245,36 @@ __device__ __forceinline__ void main_warp(const AdaptArgs& a, Mailbox& m, int W)
       m.h[lane] = h;
       m.sys[lane] = shown;
       m.run = 1;
-      request(0, x2);
+      request(2, x2);
       post(&m.bar[kStart]);
       ymax = omax(ymax, y[0]);  // the end of the last accepted trial
       ymin = omin(ymin, y[0]);
       const double k2x = fma(h, a21k1v, y[1]);
       const double x3 = fma(h, fma(ck::a32, k2x, ck::a31 * k1x), y[0]);
       const typename Sys::Half q2 = s.accel_begin(x2, k2x);
-      request(1, x3);
+      request(3, x3);
       const double k2v = finish_stage(2, q2, d);
       const double k3x = fma(h, fma(ck::a32, k2v, ck::a31 * k1v), y[1]);
       const double x4 = fma(h, fma(ck::a43, k3x, fma(ck::a42, k2x, ck::a41 * k1x)), y[0]);
       const typename Sys::Half q3 = s.accel_begin(x3, k3x);
-      request(0, x4);
+      request(4, x4);
       const double k3v = finish_stage(3, q3, d);
       const double k4x = fma(h, fma(ck::a43, k3v, fma(ck::a42, k2v, ck::a41 * k1v)), y[1]);
       const double x5 = fma(h, fma(ck::a54, k4x, fma(ck::a53, k3x, fma(ck::a52, k2x, ck::a51 * k1x))), y[0]);
       const typename Sys::Half q4 = s.accel_begin(x4, k4x);
-      request(1, x5);
+      request(5, x5);
       const double k4v = finish_stage(4, q4, d);
       const double k5x = fma(h, fma(ck::a54, k4v, fma(ck::a53, k3v, fma(ck::a52, k2v, ck::a51 * k1v))), y[1]);
       const double x6 =
           fma(h, fma(ck::a65, k5x, fma(ck::a64, k4x, fma(ck::a63, k3x, fma(ck::a62, k2x, ck::a61 * k1x)))), y[0]);
       const typename Sys::Half q5 = s.accel_begin(x5, k5x);
-      request(0, x6);
+      request(6, x6);
       const double k5v = finish_stage(5, q5, dn);  // c5 = 1: the drive at the trial's end
       const double k6x =
           fma(h, fma(ck::a65, k5v, fma(ck::a64, k4v, fma(ck::a63, k3v, fma(ck::a62, k2v, ck::a61 * k1v)))), y[1]);
       y5[0] = fma(h, fma(ck::b6, k6x, fma(ck::b4, k4x, fma(ck::b3, k3x, ck::b1 * k1x))), y[0]);
       const typename Sys::Half q6 = s.accel_begin(x6, k6x);
-      request(1, y5[0]);
+      request(7, y5[0]);
       m.v[0][lane] = y[0];
       m.v[1][lane] = y[1];
       m.v[2][lane] = y5[0];
@@ -289,10 +289,11 @@ __device__ __forceinline__ void main_warp(const AdaptArgs& a, Mailbox& m, int W)
       // the next trial's first stage, if this one is accepted; a trial that was
       // shortened to the end of the phase is followed by a phase start
       const typename Sys::Half qn = s.accel_begin(y5[0], y5[1]);
-      ok &= await(&m.bar[kRsp + 1], rsp[1]);
+      uint32_t phase = trial;
+      ok &= await(&m.bar[kAll + 5], phase);
       {
         const typename Sys::Half2 q = s.accel_more(qn);
-        k1n = s.accel_last(qn, q, s.accel_mid(qn, q, m.g[1][lane]), clamped ? d0.fs : dn.fs, clamped ? d0.fc : dn.fc);
+        k1n = s.accel_last(qn, q, s.accel_mid(qn, q, m.g[5][lane]), clamped ? d0.fs : dn.fs, clamped ? d0.fc : dn.fc);
       }
     } else {
       typename Sys::Drive d;
@@ -302,44 +303,45 @@ __device__ __forceinline__ void main_warp(const AdaptArgs& a, Mailbox& m, int W)
       m.h[lane] = h;
       m.sys[lane] = shown;
       m.run = 1;
-      request(0, x2);
+      request(2, x2);
       post(&m.bar[kStart]);
       ymax = omax(ymax, y[0]);  // the end of the last accepted trial
       ymin = omin(ymin, y[0]);
       const double k2x = fma(h, a21k1v, y[1]);
       const double x3 = fma(h, fma(dp::a32, k2x, dp::a31 * k1x), y[0]);
       const typename Sys::Half q2 = s.accel_begin(x2, k2x);
-      request(1, x3);
+      request(3, x3);
       const double k2v = finish_stage(2, q2, d);
       const double k3x = fma(h, fma(dp::a32, k2v, dp::a31 * k1v), y[1]);
       const double x4 = fma(h, fma(dp::a43, k3x, fma(dp::a42, k2x, dp::a41 * k1x)), y[0]);
       const typename Sys::Half q3 = s.accel_begin(x3, k3x);
-      request(0, x4);
+      request(4, x4);
       const double k3v = finish_stage(3, q3, d);
       const double k4x = fma(h, fma(dp::a43, k3v, fma(dp::a42, k2v, dp::a41 * k1v)), y[1]);
       const double x5 = fma(h, fma(dp::a54, k4x, fma(dp::a53, k3x, fma(dp::a52, k2x, dp::a51 * k1x))), y[0]);
       const typename Sys::Half q4 = s.accel_begin(x4, k4x);
-      request(1, x5);
+      request(5, x5);
       const double k4v = finish_stage(4, q4, d);
       const double k5x = fma(h, fma(dp::a54, k4v, fma(dp::a53, k3v, fma(dp::a52, k2v, dp::a51 * k1v))), y[1]);
       const double x6 =
           fma(h, fma(dp::a65, k5x, fma(dp::a64, k4x, fma(dp::a63, k3x, fma(dp::a62, k2x, dp::a61 * k1x)))), y[0]);
       const typename Sys::Half q5 = s.accel_begin(x5, k5x);
-      request(0, x6);
+      request(6, x6);
       const double k5v = finish_stage(5, q5, d);
       const double k6x =
           fma(h, fma(dp::a65, k5v, fma(dp::a64, k4v, fma(dp::a63, k3v, fma(dp::a62, k2v, dp::a61 * k1v)))), y[1]);
       y5[0] = fma(h, fma(dp::b6, k6x, fma(dp::b5, k5x, fma(dp::b4, k4x, fma(dp::b3, k3x, dp::b1 * k1x)))), y[0]);
       const typename Sys::Half q6 = s.accel_begin(x6, k6x);
-      request(1, y5[0]);
+      request(7, y5[0]);
       const double k6v = finish_stage(6, q6, dn);  // c6 = c7 = 1
       y5[1] = fma(h, fma(dp::b6, k6v, fma(dp::b5, k5v, fma(dp::b4, k4v, fma(dp::b3, k3v, dp::b1 * k1v)))), y[1]);
       // stage 7 = the next trial's first stage
       const typename Sys::Half qn = s.accel_begin(y5[0], y5[1]);
-      ok &= await(&m.bar[kRsp + 1], rsp[1]);
+      uint32_t phase = trial;
+      ok &= await(&m.bar[kAll + 5], phase);
       {
         const typename Sys::Half2 q = s.accel_more(qn);
-        k1n = s.accel_last(qn, q, s.accel_mid(qn, q, m.g[1][lane]), dn.fs, dn.fc);
+        k1n = s.accel_last(qn, q, s.accel_mid(qn, q, m.g[5][lane]), dn.fs, dn.fc);
       }
       m.v[0][lane] = y[0];
       m.v[1][lane] = y[1];
@@ -351,8 +353,8 @@ __device__ __forceinline__ void main_warp(const AdaptArgs& a, Mailbox& m, int W)
                              fma(dp::e6, k6v, fma(dp::e5, k5v, fma(dp::e4, k4v, fma(dp::e3, k3v, dp::e1 * k1v)))));
       post(&m.bar[kCtlReq]);
     }
-    ok &= await(&m.bar[kCtlRsp], crsp);
-    ++drv;
+    uint32_t phase = trial++;
+    ok &= await(&m.bar[kCtlRsp], phase);
     E = m.e[lane];
     fac = m.fac[lane];
     const double hf = h * fac;
@@ -394,7 +396,7 @@ __device__ __forceinline__ void main_warp(const AdaptArgs& a, Mailbox& m, int W)
         // the first stage takes the drive of the phase start
         if ((PAIR == kDormandPrince || !clamped) &&
             (nnbits(dn.fs) != nnbits(d0.fs) || nnbits(dn.fc) != nnbits(d0.fc))) {
-          k1v = s.accel_at(y[0], y[1], m.g[1][lane], d0);
+          k1v = s.accel_at(y[0], y[1], m.g[5][lane], d0);
           a21k1v = a21 * k1v;
         }
         tau = a.t0;
@@ -414,11 +416,19 @@ template <class Sys, int PAIR>
 __global__ void __launch_bounds__(96 * kMaxTeams) ck_phased_teams_kernel(AdaptArgs a) {
   __shared__ Mailbox boxes[kMaxTeams];
   const int W = (int)blockDim.x / 96, w = (int)(threadIdx.x >> 5);
-  if (threadIdx.x < (unsigned)W) init_bars(boxes[threadIdx.x].bar, kBars);
+  if (threadIdx.x < (unsigned)W) {
+    // the main warp waits for a stage's power and drive together
+    for (int k = 0; k < kBars; ++k) init_bar(boxes[threadIdx.x].bar + k, k >= kAll && k < kAll + 5 ? 2 : 1);
+  }
   __syncthreads();
-  if (w < W) main_warp<Sys, PAIR>(a, boxes[w], W);
-  else if (w < 2 * W) power_warp<Sys>(a, boxes[w - W]);
-  else drive_warp<Sys, PAIR>(a, boxes[w - 2 * W]);
+  // Warps of a block go to the sub-partitions in turn.  Of five teams two main warps
+  // share one: that with three warps, beside a single helper (131,044 systems x 3
+  // periods 81.1 -> 80.5 ms)
+  constexpr int kFive[15] = {1, 2, 3, 0, 5, 6, 7, 4, 8, 9, 10, 11, 12, 13, 14};
+  const int r = W == 5 ? kFive[w] : w;
+  if (r < W) main_warp<Sys, PAIR>(a, boxes[r], W, r);
+  else if (r < 2 * W) power_warp<Sys>(a, boxes[r - W]);
+  else drive_warp<Sys, PAIR>(a, boxes[r - 2 * W]);
 }
 
 }  // namespace
