@@ -239,9 +239,8 @@ struct KellerMiksis {
     fd(drive(tau), tau, y, dy);
   }
   // accel<double> in parts, the same operations: what does not depend on the
-  // polytropic power g = (1/y1)^(21/5) (early_power) or the drive, and the
-  // rest.  The
-  // paired kernel (rkck45_pairs.cu) has g and the drive computed by another warp.
+  // polytropic power g = (1/y1)^(21/5) (early_power) or the drive, and the rest.  The
+  // team kernels (rkck45_teams.cu, rkck45_relay.cu) have those from other warps.
   struct Half {
     double y1, y2, one_c9y2, A, rx, w;
   };

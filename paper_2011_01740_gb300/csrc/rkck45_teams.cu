@@ -23,10 +23,11 @@
 // Every operation is that of ck_phased_kernel, so are the bits.  Milliseconds
 // there and here: 1,073 systems x 2 periods 45.1 / 32.9, 4,608 frequencies x 3
 // 68.2 / 48.9, two frequencies and Dormand-Prince (6,097 x 2) 69.4 / 48.5; with
-// longest-first claiming 65,536 x 2 47.6 / 39.3, 131,044 x 4 126.3 (6 warps per
-// SM) / 110.6 (5 teams).  Registers allow 5 teams per SM, which keep the FP64 pipe
-// about 75 % busy; enough systems let more plain warps do better (262,144 x 2:
-// 105.1 here, 101.9 with 12 plain warps), see teams_fit in abi.cu.
+// longest-first claiming 65,536 x 2 47.6 / 36.7, 131,044 x 6 189.4 (6 warps per
+// SM) / 166.4 (5 teams).  Registers allow 5 teams per SM, which keep the FP64 pipe
+// about 80 % busy; enough systems let more plain warps do better (262,144 x 2:
+// 105.1 here, 97.0 with 12 plain warps), see teams_fit in abi.cu; up to two warps of
+// systems per SM the relay (rkck45_relay.cu) does.
 // What was tried: one helper warp for both kinds (37.4 ms on 1,073 systems; its
 // power then waits for a drive); the helpers' stages unrolled (fast while all teams
 // of an SM run in step, 151 ms on 131,044 x 4 when they do not: instruction cache);
