@@ -22,6 +22,7 @@ cudaError_t launch_ck45_df_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch
 cudaError_t launch_ck45_df_events(const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_relay(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
+cudaError_t launch_ck45_events_relay(const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_spt2(int sys, unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_order(const int64_t* steps, int64_t n, int32_t* order, unsigned* hist,
                          cudaStream_t s);
@@ -122,7 +123,7 @@ ens_status cuda_fail(ens_ctx* c, cudaError_t e, const char* what) {
 //   launch earlier, as four teams of three warps do not fit (19,200 x 2: 40.8 / 29.2).
 //   Valves take about the same number of steps each, and neighbours take them
 //   alike, which claiming by cost breaks up: plain launches of 1 warp a block
-//   (1,000: 21.5 / 25.4; 32,768: 25.8 / 37.2; 65,536: 46.4 / 60.7; 262,144: 168 /
+//   (1,000: 17.0, in one warp a trial 21.5 / 25.4; 32,768: 25.8 / 37.2; 65,536: 46.4 / 60.7; 262,144: 168 /
 //   211; 2 warps a block 21.4, 28.2, 46.7 and 170); double-float ones of 8, whose
 //   warps share the fetch of a long trial (65,536: 20.8, 1 warp a block 21.8; 524,288:
 //   132 / 136; persistent 5 warps per SM 282).
@@ -256,6 +257,14 @@ bool relay_fits(const ens_ctx* c, AdaptLaunch L) {
   return teams_fit(c, L) && L.grid * (L.block / 32) <= 2 * (int64_t)c->sm_count;
 }
 
+// Whether the valves of an FP64 Cash-Karp launch run in relays (valve_relay.cu): blocks
+// of one warp of systems, up to the four per SM that fit (1,000 valves x 16 time units
+// 21.4 -> 16.8 ms, 19,456 21.6 -> 20.1).
+bool valve_relay_fits(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L) {
+  return c->sys == ENS_SYS_RELIEF_VALVE && a.n_phases == 0 && a.pair == kCashKarp && L.spt == 1 && L.block == 32 &&
+         L.grid <= 4 * (int64_t)c->sm_count;
+}
+
 // The same for double-float phases, in teams of two (df64.cu): up to 6 per SM
 // (131,044 systems x 2 periods 41.9 ms against 45.4 in plain warps; 262,144 x 2
 // 83.7 against 62.1 in 12 plain warps per SM).
@@ -271,6 +280,7 @@ cudaError_t launch_adaptive(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L,
     return df_teams_fit(c, L) ? launch_ck45_df_teams(c->km_flags, a, L, s) : launch_ck45_df(c->km_flags, a, L, s);
   }
   if (L.spt == 2) return launch_ck45_spt2(c->sys, c->km_flags, a, L, s);
+  if (valve_relay_fits(c, a, L)) return launch_ck45_events_relay(a, L, s);
   if (relay_fits(c, L)) return launch_ck45_relay(c->km_flags, a, AdaptLaunch{L.grid * (L.block / 32), 32}, s);
   if (teams_fit(c, L)) return launch_ck45_teams(c->km_flags, a, L, s);
   return launch_ck45(c->sys, c->km_flags, a, L, s);
