@@ -142,6 +142,7 @@ ens_launch default_launch(const ens_ctx* c) {
   const bool teams = has_teams(c), dual_df = c->tol.prec == ENS_FP32X2 && (c->km_flags & kKmDual);
   if (c->n <= (int64_t)c->sm_count * (teams || dual_df ? 64 : 128)) {
     if (c->tol.prec == ENS_FP32X2) L.block = 64;  // 16,384 x 2: 33.0, one warp a block 35.7
+    if (c->tol.prec == ENS_FP64 && !teams) L.block = 128;  // exponent 3.99, 16,384 x 1: 49.6, one warp a block 52.0
     return L;
   }
   L.mode = ENS_LAUNCH_PERSISTENT;
@@ -269,7 +270,7 @@ bool valve_relay_fits(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L) {
 // (131,044 systems x 2 periods 41.9 ms against 45.4 in plain warps; 262,144 x 2
 // 83.7 against 62.1 in 12 plain warps per SM).
 bool df_teams_fit(const ens_ctx* c, AdaptLaunch L) {
-  return L.block <= 192 && L.grid * (L.block / 32) <= 6 * (int64_t)c->sm_count;
+  return L.block <= 256 && L.grid * (L.block / 32) <= (L.block <= 192 ? 6 : 8) * (int64_t)c->sm_count;
 }
 
 // the adaptive kernel of the context's precision
@@ -354,10 +355,12 @@ AdaptLaunch adapt_launch(const ens_ctx* c, const ens_launch& L) {
 // of the horizon) of every system in plain mode, then the systems sorted by
 // decreasing pilot step count into c->order.  The pilot only ranks the
 // systems (the claim order never changes what a system computes), so it runs at
-// a tolerance of at least kPilotTol, a tenth of the steps of a 1e-10 pilot,
-// and Keller-Miksis phases are ranked in split precision: a trial of the
+// a tolerance of at least kPilotTol, and Keller-Miksis phases are ranked at
+// kPhasePilotTol in split precision: a trial of the
 // longest system, which bounds the pilot, takes 2.9 us there against 10.4 us
 // in FP64 (131,044 systems: pilot and sort 1.6 ms, at 1e-7 in FP64 14).
+// The tangent system keeps a pilot of its own: its steps follow the tangent vector too
+// (131,044 x 2 periods 173 ms, ranked by the plain system 240).
 // kPilotTrials bounds a system whose float pilot would be held up by rounding; it
 // ranks with the longest.
 ens_status enqueue_order(ens_ctx* c, const AdaptArgs& a, cudaStream_t s) {
@@ -371,11 +374,13 @@ ens_status enqueue_order(ens_ctx* c, const AdaptArgs& a, cudaStream_t s) {
   } else {
     p.t1 = p.t0 + (p.t1 - p.t0) / 16.0;
   }
-  p.rtol = p.rtol > kPilotTol ? p.rtol : kPilotTol;
-  p.atol = p.atol > kPilotTol ? p.atol : kPilotTol;
+  const bool split = c->sys == ENS_SYS_KELLER_MIKSIS && p.n_phases > 0;
+  const double loosest = split ? kPhasePilotTol : kPilotTol;
+  p.rtol = std::max(p.rtol, loosest);
+  p.atol = std::max(p.atol, loosest);
   AdaptLaunch PL{(c->n + 127) / 128, 128};
   cudaError_t e;
-  if (is_km(c->sys) && p.n_phases > 0) {
+  if (split) {
     p.max_steps = std::min<int64_t>(p.max_steps, kPilotTrials);
     e = launch_ck45_fp32c(c->km_flags, p, PL, s);
   } else {

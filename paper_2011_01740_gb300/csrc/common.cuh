@@ -163,16 +163,17 @@ constexpr double e1 = b1 - 5179.0 / 57600.0, e3 = b3 - 7571.0 / 16695.0, e4 = b4
 // Embedded Runge-Kutta pair of the adaptive kernels.
 enum Pair : int { kCashKarp = 0, kDormandPrince = 1 };
 
-// Loosest tolerance of the claim-order pilot.  The pilot only ranks systems by
-// their step counts, so it runs at max(tol, 1e-5), a tenth of the steps of a 1e-10
-// pilot, and the claim order never changes what a system computes.  Pilot and sort,
+// Loosest tolerance of a claim-order pilot.  The pilot only ranks systems by their
+// step counts, and the claim order never changes what a system computes, so it runs at
+// max(tol, 1e-7), a quarter of the steps of a 1e-10 pilot; that of Keller-Miksis phases
+// at max(tol, 1e-5), a tenth.  Pilot and sort,
 // and the whole pass, at 1e-7 / 1e-6 / 1e-5 / 1e-4 (milliseconds): split precision 262,144 x
 // 4 periods 3.7 / 2.7 / 2.0 / 1.6 of 23.1 / 22.0 / 21.5 / 21.0; FP64 19,200 x 2 22.9 / 22.5 /
 // 22.1 / 21.9; 131,044 x 6 170.1 / 169.8 / 170.2 / 171.8, where a coarser ranking begins to
 // cost what its pilot saves.
-constexpr double kPilotTol = 1e-5;
+constexpr double kPilotTol = 1e-7, kPhasePilotTol = 1e-5;
 // Most trials of one system in a split-precision pilot (a forcing period takes
-// the hardest systems of the p_A x f maps a few hundred at kPilotTol).
+// the hardest systems of the p_A x f maps a few hundred at kPhasePilotTol).
 constexpr int64_t kPilotTrials = 1 << 14;
 
 // Host helpers of abi.cu shared with the other entry points.

@@ -21,14 +21,15 @@ constexpr uint32_t pair_rhs(int PAIR) { return PAIR == kDormandPrince ? 6u : 5u;
 __device__ __forceinline__ double err_weight(double y, double y5, double rtol, double atol) {
   return rcp_fx(fma(rtol, nnmax(absd(y), absd(y5)), atol));
 }
-__device__ __forceinline__ double err_ratio(double err, double weight) { return absd(fmul(absd(err), weight)); }
-template <int D>
+template <class Ops = FusedOps>
+__device__ __forceinline__ double err_ratio(double err, double weight) { return absd(Ops::mul(absd(err), weight)); }
+template <int D, class Ops = FusedOps>
 __device__ __forceinline__ double err_norm(const double* y, const double* y5, const double* err,
                                            double rtol, double atol) {
   double E = 0.0;
 #pragma unroll
   for (int c = 0; c < D; ++c) {
-    E = nnmax(E, err_ratio(err[c], err_weight(y[c], y5[c], rtol, atol)));
+    E = nnmax(E, err_ratio<Ops>(err[c], err_weight(y[c], y5[c], rtol, atol)));
   }
   return E;
 }
@@ -39,10 +40,11 @@ __device__ __forceinline__ bool accept(double E) { return nnbits(E) <= nnbits(1.
 // E > 4.5^5 = 1845.3 and E < 0.18^5 = 1.9e-4, so E is clamped to [1e-4, 2000]
 // first (same result, and keeps the float seed of inv_fifth_root_fx in range).
 // E >= 0 or NaN as err_norm returns it.
+template <class Ops = FusedOps>
 __device__ __forceinline__ double step_factor(double E) {
   if (nnbits(E) > nnbits(__longlong_as_double(0x7ff0000000000000LL))) return 0.2;  // NaN
   const double Ec = nnmin(nnmax(E, 1e-4), 2000.0);
-  const double fac = fmul(0.9, inv_fifth_root_fx(Ec));
+  const double fac = Ops::mul(0.9, inv_fifth_root_fx(Ec));
   return nnmin(nnmax(fac, 0.2), 5.0);
 }
 

@@ -297,7 +297,7 @@ namespace {
 // 1,073 systems x 2 periods 41.1 -> 29.1 ms, 65,536 in 3 teams per SM 51.9 -> 42.8.
 // Four is what the registers hold; in 6 teams of two 131,044 take 70.9 ms (4 of three
 // 74.0), as the FP64 pipe then bounds both.
-constexpr int kMaxDfTeams = 6, kMaxDfTeams3 = 4;
+constexpr int kMaxDfTeams = 6, kMaxDfTeams3 = 4, kMaxDfTeams8 = 8;
 enum : int { kDfStart = 0, kDfDrive = 1, kDfBars = 6 };
 
 struct __align__(16) DfMailbox {
@@ -798,13 +798,18 @@ cudaError_t launch_ck45_df_events(const AdaptArgs& a, AdaptLaunch L, cudaStream_
 cudaError_t launch_ck45_df_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s) {
   if (a.n == 0) return cudaSuccess;
   if (a.n_phases <= 0) return cudaErrorInvalidValue;
-  if (L.grid <= 0 || L.grid > 0x7fffffffLL || L.block < 32 || L.block % 32 || L.block > 32 * kMaxDfTeams)
+  if (L.grid <= 0 || L.grid > 0x7fffffffLL || L.block < 32 || L.block % 32 || L.block > 32 * kMaxDfTeams8)
     return cudaErrorInvalidConfiguration;
   const bool dual = flags & kKmDual, three = dual && L.block <= 32 * kMaxDfTeams3;
   const dim3 g((unsigned)L.grid), b((three ? 3 : 2) * (unsigned)L.block);
   if (three) ck_phased_df_teams_kernel<true, 2, kMaxDfTeams3><<<g, b, 0, s>>>(a);
-  else if (dual) ck_phased_df_teams_kernel<true, 1, kMaxDfTeams><<<g, b, 0, s>>>(a);
-  else ck_phased_df_teams_kernel<false, 1, kMaxDfTeams><<<g, b, 0, s>>>(a);
+  else if (L.block <= 32 * kMaxDfTeams) {
+    if (dual) ck_phased_df_teams_kernel<true, 1, kMaxDfTeams><<<g, b, 0, s>>>(a);
+    else ck_phased_df_teams_kernel<false, 1, kMaxDfTeams><<<g, b, 0, s>>>(a);
+  } else {
+    if (dual) ck_phased_df_teams_kernel<true, 1, kMaxDfTeams8><<<g, b, 0, s>>>(a);
+    else ck_phased_df_teams_kernel<false, 1, kMaxDfTeams8><<<g, b, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 

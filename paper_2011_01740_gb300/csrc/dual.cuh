@@ -74,6 +74,7 @@ template <bool DUAL, bool EXP215 = false>
 struct KellerMiksisTangent : KellerMiksis<DUAL, EXP215> {
   using Base = KellerMiksis<DUAL, EXP215>;
   using Drive = typename Base::Drive;
+  using Ops = PlainOps;
   static constexpr int kDim = 4;
   static constexpr int kPhaseRows = 1;  // ln |v| at each phase end
   __device__ __forceinline__ void fd(const Drive& d, double tau, const double* y, double* dy) const {

@@ -20,4 +20,17 @@ __device__ __forceinline__ double fmul(double a, double b) { return __fma_rn(a, 
 __device__ __forceinline__ double fadd(double a, double b) { return __fma_rn(a, kOneOpaque, b); }
 __device__ __forceinline__ double fsub(double a, double b) { return __fma_rn(a, kOneOpaque, -b); }
 
+// The products and sums a system's trials take: fused ones in the kernels above, where
+// they were measured.
+struct FusedOps {
+  static __device__ __forceinline__ double mul(double a, double b) { return fmul(a, b); }
+  static __device__ __forceinline__ double add(double a, double b) { return fadd(a, b); }
+  static __device__ __forceinline__ double sub(double a, double b) { return fsub(a, b); }
+};
+struct PlainOps {
+  static __device__ __forceinline__ double mul(double a, double b) { return a * b; }
+  static __device__ __forceinline__ double add(double a, double b) { return a + b; }
+  static __device__ __forceinline__ double sub(double a, double b) { return a - b; }
+};
+
 }  // namespace ens

@@ -168,6 +168,7 @@ struct NoDrive {};
 // ---------------------------------------------------------------------------
 template <bool DUAL, bool EXP215 = false>
 struct KellerMiksis {
+  using Ops = FusedOps;
   static constexpr bool kDual = DUAL;
   static constexpr int kDim = 2;
   static constexpr int kPar = 13;
@@ -284,6 +285,7 @@ struct KellerMiksis {
 // +0), which spares the FP64 pipe a min / max per evaluation.
 // ---------------------------------------------------------------------------
 struct ReliefValve {
+  using Ops = FusedOps;
   static constexpr int kDim = 3;
   static constexpr int kPar = 5;
   static constexpr int kPhaseRows = 0;

@@ -46,38 +46,38 @@ __device__ __forceinline__ void ck_trial(const Sys& s, double t, double h, const
   double k2[D], k3[D], k4[D], k5[D], k6[D], ys[D];
   double ts;
 #pragma unroll
-  for (int c = 0; c < D; ++c) ys[c] = fma(h, fmul(ck::a21, k1[c]), y[c]);
+  for (int c = 0; c < D; ++c) ys[c] = fma(h, Sys::Ops::mul(ck::a21, k1[c]), y[c]);
   ts = fma(ck::c2, h, t);
   s.fd(s.drive(ts), ts, ys, k2);
 #pragma unroll
-  for (int c = 0; c < D; ++c) ys[c] = fma(h, fma(ck::a32, k2[c], fmul(ck::a31, k1[c])), y[c]);
+  for (int c = 0; c < D; ++c) ys[c] = fma(h, fma(ck::a32, k2[c], Sys::Ops::mul(ck::a31, k1[c])), y[c]);
   ts = fma(ck::c3, h, t);
   s.fd(s.drive(ts), ts, ys, k3);
 #pragma unroll
   for (int c = 0; c < D; ++c)
-    ys[c] = fma(h, fma(ck::a43, k3[c], fma(ck::a42, k2[c], fmul(ck::a41, k1[c]))), y[c]);
+    ys[c] = fma(h, fma(ck::a43, k3[c], fma(ck::a42, k2[c], Sys::Ops::mul(ck::a41, k1[c]))), y[c]);
   ts = fma(ck::c4, h, t);
   s.fd(s.drive(ts), ts, ys, k4);
 #pragma unroll
   for (int c = 0; c < D; ++c)
-    ys[c] = fma(h, fma(ck::a54, k4[c], fma(ck::a53, k3[c], fma(ck::a52, k2[c], fmul(ck::a51, k1[c])))),
+    ys[c] = fma(h, fma(ck::a54, k4[c], fma(ck::a53, k3[c], fma(ck::a52, k2[c], Sys::Ops::mul(ck::a51, k1[c])))),
                 y[c]);
-  ts = fadd(t, h);  // c5 = 1
+  ts = Sys::Ops::add(t, h);  // c5 = 1
   d5 = s.drive(ts);
   s.fd(d5, ts, ys, k5);
 #pragma unroll
   for (int c = 0; c < D; ++c)
     ys[c] = fma(h,
                 fma(ck::a65, k5[c],
-                    fma(ck::a64, k4[c], fma(ck::a63, k3[c], fma(ck::a62, k2[c], fmul(ck::a61, k1[c]))))),
+                    fma(ck::a64, k4[c], fma(ck::a63, k3[c], fma(ck::a62, k2[c], Sys::Ops::mul(ck::a61, k1[c]))))),
                 y[c]);
   ts = fma(ck::c6, h, t);
   s.fd(s.drive(ts), ts, ys, k6);
 #pragma unroll
   for (int c = 0; c < D; ++c) {
-    y5[c] = fma(h, fma(ck::b6, k6[c], fma(ck::b4, k4[c], fma(ck::b3, k3[c], fmul(ck::b1, k1[c])))), y[c]);
-    err[c] = fmul(h, fma(ck::d6, k6[c],
-                     fma(ck::d5, k5[c], fma(ck::d4, k4[c], fma(ck::d3, k3[c], fmul(ck::d1, k1[c]))))));
+    y5[c] = fma(h, fma(ck::b6, k6[c], fma(ck::b4, k4[c], fma(ck::b3, k3[c], Sys::Ops::mul(ck::b1, k1[c])))), y[c]);
+    err[c] = Sys::Ops::mul(h, fma(ck::d6, k6[c],
+                     fma(ck::d5, k5[c], fma(ck::d4, k4[c], fma(ck::d3, k3[c], Sys::Ops::mul(ck::d1, k1[c]))))));
   }
 }
 
@@ -94,21 +94,21 @@ __device__ __forceinline__ void dp_trial(const Sys& s, double t, double h, const
   double k2[D], k3[D], k4[D], k5[D], k6[D], ys[D];
   double ts;
 #pragma unroll
-  for (int c = 0; c < D; ++c) ys[c] = fma(h, fmul(dp::a21, k1[c]), y[c]);
+  for (int c = 0; c < D; ++c) ys[c] = fma(h, Sys::Ops::mul(dp::a21, k1[c]), y[c]);
   ts = fma(dp::c2, h, t);
   s.fd(s.drive(ts), ts, ys, k2);
 #pragma unroll
-  for (int c = 0; c < D; ++c) ys[c] = fma(h, fma(dp::a32, k2[c], fmul(dp::a31, k1[c])), y[c]);
+  for (int c = 0; c < D; ++c) ys[c] = fma(h, fma(dp::a32, k2[c], Sys::Ops::mul(dp::a31, k1[c])), y[c]);
   ts = fma(dp::c3, h, t);
   s.fd(s.drive(ts), ts, ys, k3);
 #pragma unroll
   for (int c = 0; c < D; ++c)
-    ys[c] = fma(h, fma(dp::a43, k3[c], fma(dp::a42, k2[c], fmul(dp::a41, k1[c]))), y[c]);
+    ys[c] = fma(h, fma(dp::a43, k3[c], fma(dp::a42, k2[c], Sys::Ops::mul(dp::a41, k1[c]))), y[c]);
   ts = fma(dp::c4, h, t);
   s.fd(s.drive(ts), ts, ys, k4);
 #pragma unroll
   for (int c = 0; c < D; ++c)
-    ys[c] = fma(h, fma(dp::a54, k4[c], fma(dp::a53, k3[c], fma(dp::a52, k2[c], fmul(dp::a51, k1[c])))),
+    ys[c] = fma(h, fma(dp::a54, k4[c], fma(dp::a53, k3[c], fma(dp::a52, k2[c], Sys::Ops::mul(dp::a51, k1[c])))),
                 y[c]);
   ts = fma(dp::c5, h, t);
   s.fd(s.drive(ts), ts, ys, k5);
@@ -116,23 +116,23 @@ __device__ __forceinline__ void dp_trial(const Sys& s, double t, double h, const
   for (int c = 0; c < D; ++c)
     ys[c] = fma(h,
                 fma(dp::a65, k5[c],
-                    fma(dp::a64, k4[c], fma(dp::a63, k3[c], fma(dp::a62, k2[c], fmul(dp::a61, k1[c]))))),
+                    fma(dp::a64, k4[c], fma(dp::a63, k3[c], fma(dp::a62, k2[c], Sys::Ops::mul(dp::a61, k1[c]))))),
                 y[c]);
-  ts = fadd(t, h);  // c6 = c7 = 1
+  ts = Sys::Ops::add(t, h);  // c6 = c7 = 1
   d7 = s.drive(ts);
   s.fd(d7, ts, ys, k6);
 #pragma unroll
   for (int c = 0; c < D; ++c)
     y5[c] = fma(h,
                 fma(dp::b6, k6[c],
-                    fma(dp::b5, k5[c], fma(dp::b4, k4[c], fma(dp::b3, k3[c], fmul(dp::b1, k1[c]))))),
+                    fma(dp::b5, k5[c], fma(dp::b4, k4[c], fma(dp::b3, k3[c], Sys::Ops::mul(dp::b1, k1[c]))))),
                 y[c]);
   s.fd(d7, ts, y5, k7);
 #pragma unroll
   for (int c = 0; c < D; ++c)
-    err[c] = fmul(h, fma(dp::e7, k7[c],
+    err[c] = Sys::Ops::mul(h, fma(dp::e7, k7[c],
                      fma(dp::e6, k6[c],
-                         fma(dp::e5, k5[c], fma(dp::e4, k4[c], fma(dp::e3, k3[c], fmul(dp::e1, k1[c])))))));
+                         fma(dp::e5, k5[c], fma(dp::e4, k4[c], fma(dp::e3, k3[c], Sys::Ops::mul(dp::e1, k1[c])))))));
 }
 
 // One trial of the selected pair.  dn receives the drive at t + h; for
@@ -228,7 +228,7 @@ __global__ void __launch_bounds__(256) ck_phased_kernel(AdaptArgs a) {
     } else {
       double h = dt;
       bool clamped = false;
-      const double rest = fsub(tau_end, tau);  // > 0 inside a phase
+      const double rest = Sys::Ops::sub(tau_end, tau);  // > 0 inside a phase
       if (nnbits(h) >= nnbits(rest)) {
         h = rest;
         clamped = true;
@@ -241,10 +241,10 @@ __global__ void __launch_bounds__(256) ck_phased_kernel(AdaptArgs a) {
       pair_trial<PAIR>(s, tau, h, y, k1, y5, err, kn, d5);
       nrhs += pair_rhs(PAIR);
       ++trials;
-      const double E = err_norm<D>(y, y5, err, a.rtol, a.atol);
-      const double fac = step_factor(E);
+      const double E = err_norm<D, typename Sys::Ops>(y, y5, err, a.rtol, a.atol);
+      const double fac = step_factor<typename Sys::Ops>(E);
       if (accept(E)) {
-        tau = clamped ? tau_end : fadd(tau, h);
+        tau = clamped ? tau_end : Sys::Ops::add(tau, h);
         dk = d5;  // drive at tau + h; a phase end below resets it
 #pragma unroll
         for (int c = 0; c < D; ++c) {
@@ -376,7 +376,7 @@ __global__ void __launch_bounds__(128) ck_phased2_kernel(AdaptArgs a) {
       }
       L.h = L.dt;
       L.clamped = false;
-      const double rest = fsub(tau_end, L.tau);
+      const double rest = Sys::Ops::sub(tau_end, L.tau);
       if (nnbits(L.h) >= nnbits(rest)) {
         L.h = rest;
         L.clamped = true;
@@ -388,8 +388,8 @@ __global__ void __launch_bounds__(128) ck_phased2_kernel(AdaptArgs a) {
       PhaseSlot<Sys>& L = S[q];
       L.s.fd(L.dk, L.tau, L.y, L.k1);
       ck_trial(L.s, L.tau, L.h, L.y, L.k1, L.y5, L.err, L.d5);
-      L.E = err_norm<D>(L.y, L.y5, L.err, a.rtol, a.atol);
-      L.fac = step_factor(L.E);
+      L.E = err_norm<D, typename Sys::Ops>(L.y, L.y5, L.err, a.rtol, a.atol);
+      L.fac = step_factor<typename Sys::Ops>(L.E);
     }
     // per slot: the outcome
 #pragma unroll
@@ -415,7 +415,7 @@ __global__ void __launch_bounds__(128) ck_phased2_kernel(AdaptArgs a) {
         L.nrhs += pair_rhs(kCashKarp);
         ++L.trials;
         if (accept(L.E)) {
-          L.tau = L.clamped ? tau_end : fadd(L.tau, L.h);
+          L.tau = L.clamped ? tau_end : Sys::Ops::add(L.tau, L.h);
           L.dk = L.d5;
 #pragma unroll
           for (int c = 0; c < D; ++c) L.y[c] = L.y5[c];
@@ -546,7 +546,7 @@ __global__ void __launch_bounds__(256) ck_events_kernel(AdaptArgs a) {
     } else {
       double h = dt;
       int limited = 0;
-      const double rest = fsub(a.t1, t);  // > 0 before the end
+      const double rest = Sys::Ops::sub(a.t1, t);  // > 0 before the end
       if (nnbits(h) >= nnbits(rest)) {
         h = rest;
         limited = 1;
@@ -563,8 +563,8 @@ __global__ void __launch_bounds__(256) ck_events_kernel(AdaptArgs a) {
       pair_trial<PAIR>(s, t, h, y, k1, y5, err, kn, d5);
       nrhs += pair_rhs(PAIR);
       ++trials;
-      const double E = err_norm<D>(y, y5, err, a.rtol, a.atol);
-      const double fac = step_factor(E);
+      const double E = err_norm<D, typename Sys::Ops>(y, y5, err, a.rtol, a.atol);
+      const double fac = step_factor<typename Sys::Ops>(E);
       if (!accept(E)) {
         ++nrej;
         dt = h * fac;
@@ -595,7 +595,7 @@ __global__ void __launch_bounds__(256) ck_events_kernel(AdaptArgs a) {
             y[c] = y5[c];
             if (PAIR == kDormandPrince) k1[c] = kn[c];
           }
-          t = (limited == 1) ? a.t1 : fadd(t, h);
+          t = (limited == 1) ? a.t1 : Sys::Ops::add(t, h);
           k1v = PAIR == kDormandPrince;  // k7 = f(t + h, y5); the impact law clears it
           ++nacc;
           ev_retries = 0;
@@ -681,7 +681,7 @@ __global__ void __launch_bounds__(256) ck_plain_kernel(AdaptArgs a) {
     } else {
       double h = dt;
       bool clamped = false;
-      const double rest = fsub(a.t1, t);  // > 0 before the end
+      const double rest = Sys::Ops::sub(a.t1, t);  // > 0 before the end
       if (nnbits(h) >= nnbits(rest)) {
         h = rest;
         clamped = true;
@@ -694,10 +694,10 @@ __global__ void __launch_bounds__(256) ck_plain_kernel(AdaptArgs a) {
       pair_trial<PAIR>(s, t, h, y, k1, y5, err, kn, d5);
       nrhs += pair_rhs(PAIR);
       ++trials;
-      const double E = err_norm<D>(y, y5, err, a.rtol, a.atol);
-      const double fac = step_factor(E);
+      const double E = err_norm<D, typename Sys::Ops>(y, y5, err, a.rtol, a.atol);
+      const double fac = step_factor<typename Sys::Ops>(E);
       if (accept(E)) {
-        t = clamped ? a.t1 : fadd(t, h);
+        t = clamped ? a.t1 : Sys::Ops::add(t, h);
         dk = d5;  // t + h; a clamped step ends the system
 #pragma unroll
         for (int c = 0; c < D; ++c) {
@@ -726,6 +726,7 @@ __global__ void __launch_bounds__(256) ck_plain_kernel(AdaptArgs a) {
 template <class Fixed>
 struct AdaptFixed : Fixed {
   using Drive = NoDrive;
+  using Ops = PlainOps;
   __device__ __forceinline__ void f(double t, const double* y, double* dy) const {
     Fixed::template f<false>(t, y, dy);
   }

@@ -14,7 +14,7 @@ pytestmark = pytest.mark.gpu
 READ = (ens.ENS_STATE, ens.ENS_ACC, ens.ENS_STATUS, ens.ENS_NSTEPS, ens.ENS_NREJ, ens.ENS_NRHS, ens.ENS_TIME,
         ens.ENS_DT)
 PLAIN, PERSISTENT = ens.ENS_LAUNCH_PLAIN, ens.ENS_LAUNCH_PERSISTENT
-ONE_WARP = dict(mode=PLAIN, block=256, blocks_per_sm=0)        # blocks above 160 (192) threads: no teams
+ONE_WARP = dict(mode=PLAIN, block=256, blocks_per_sm=0)        # FP64 blocks above 160 threads: no teams
 
 
 def _solve(ctx, **launch):
@@ -32,11 +32,18 @@ def _compare(n, launch, solver=ens.ENS_RKCK45, dual=False, t0=0.0, **tol):
     C = ens.ens_km_coefficients(*[ph[k] for k in ("pA1", "f1", "pA2", "f2", "theta", "RE")], km["liquid"])
     assert np.any(C[6]) == dual
     t = ens.make_tol(**{**dict(rtol=1e-8, atol=1e-8, n_phases=3), **tol})
-    ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS, n, C, km["y0"], (t0, t0 + 1.0), solver, t)
-    try:
-        ref, got = _solve(ctx, **ONE_WARP), _solve(ctx, **launch)
-    finally:
-        ens.ens_destroy(ctx)
+    # the double-float one-warp kernel takes launches of more than 8 warps per SM
+    copies = -(-40000 // n) if t.prec == ens.ENS_FP32X2 else 1
+    out = []
+    for reps, shape in ((copies, ONE_WARP), (1, launch)):
+        ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS, n * reps, np.tile(C, (1, reps)), np.tile(km["y0"], (1, reps)),
+                             (t0, t0 + 1.0), solver, t)
+        try:
+            r = _solve(ctx, **shape)
+        finally:
+            ens.ens_destroy(ctx)
+        out.append([r[0]] + [a[..., :n] for a in r[1:]])
+    ref, got = out
     assert ref[0] == got[0]
     for w, a, b in zip(READ, ref[1:], got[1:]):
         assert np.array_equal(a, b, equal_nan=True), w
@@ -62,7 +69,9 @@ def test_teams_give_the_one_warp_bits(n, launch, solver, dual):
 @pytest.mark.parametrize("n,launch", [
     (1, dict(mode=PLAIN, block=32, blocks_per_sm=0)),
     (193, dict(mode=PLAIN, block=192, blocks_per_sm=0)),
+    (257, dict(mode=PLAIN, block=256, blocks_per_sm=0)),
     (23000, dict(mode=PERSISTENT, block=128, blocks_per_sm=1, cost_order=0)),
+    (60000, dict(mode=PERSISTENT, block=224, blocks_per_sm=1, cost_order=1)),
     (60000, dict(mode=PERSISTENT, block=192, blocks_per_sm=1, cost_order=1)),
     (30000, dict(mode=PERSISTENT, block=64, blocks_per_sm=3, cost_order=1)),
 ])
