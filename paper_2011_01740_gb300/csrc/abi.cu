@@ -266,7 +266,8 @@ bool valve_relay_fits(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L) {
          L.grid <= 4 * (int64_t)c->sm_count;
 }
 
-// The same for double-float phases, in teams of two (df64.cu): up to 6 per SM
+// The same for double-float phases, in teams of two or three (df64.cu): up to 6 per
+// SM, 8 in larger blocks (8 warps per SM, 131,044 x 2: 42.3 ms, plain 49.0)
 // (131,044 systems x 2 periods 41.9 ms against 45.4 in plain warps; 262,144 x 2
 // 83.7 against 62.1 in 12 plain warps per SM).
 bool df_teams_fit(const ens_ctx* c, AdaptLaunch L) {

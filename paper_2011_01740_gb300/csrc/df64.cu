@@ -793,8 +793,8 @@ cudaError_t launch_ck45_df_events(const AdaptArgs& a, AdaptLaunch L, cudaStream_
   return cudaGetLastError();
 }
 
-// An adaptive launch of L.block systems per block in teams of two warps, at most
-// 192 systems a block.
+// An adaptive launch of L.block systems per block in teams of two or three warps, at
+// most 256 systems a block.
 cudaError_t launch_ck45_df_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s) {
   if (a.n == 0) return cudaSuccess;
   if (a.n_phases <= 0) return cudaErrorInvalidValue;
