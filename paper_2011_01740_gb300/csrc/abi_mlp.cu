@@ -279,9 +279,11 @@ ens_status set_smem_attrs(ens_mlp* m) {
 // A feature 2 (log v - l0) / (l1 - l0) - 1, rounded to float.  Logarithm and division
 // in FP64 held the FP64 pipe for 75 instructions a point (4.2 M points: 665 us);
 // double-float pairs (df.cuh) on the FP32 pipes give the value to within 2^-42 of
-// its terms, and the float that it rounds to is the FP64 formula's unless a rounding
-// boundary lies within twice that.  Then, and for v that is not positive and
-// normal, the FP64 formula decides.
+// its terms and s 2^-47, s = 2 / (l1 - l0): a pair cuts the mantissa m of v below 2^-47,
+// which log v takes over whatever its own size.  The float that the value rounds to is
+// the FP64 formula's unless a rounding boundary lies within twice that.  Then, and for v
+// that is not positive and normal, the FP64 formula decides: for nearly all points of a
+// range narrower than 1e-7.
 struct LogFeature {
   double l0, l1;
   df::DF l0p, scale;   // l0 and 2 / (l1 - l0) as pairs
@@ -291,7 +293,7 @@ struct LogFeature {
     l0p = df::from_double(a);
     scale = df::from_double(s);
     per_log = 0x1p-41f * (float)s;
-    margin = 0x1p-41f * (2.0f + (float)(s * fabs(a)));
+    margin = 0x1p-41f * (2.0f + (float)(s * fabs(a))) + 0x1p-46f * (float)s;
   }
   __device__ __forceinline__ float operator()(double v) const {
     using namespace df;
