@@ -287,7 +287,15 @@ cudaError_t launch_adaptive(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L,
   if (L.spt == 2) return launch_ck45_spt2(c->sys, c->km_flags, a, L, s);
   if (valve_relay_fits(c, a, L)) return launch_ck45_events_relay(a, L, s);
   if (relay_fits(c, L)) return launch_ck45_relay(c->km_flags, a, AdaptLaunch{L.grid * (L.block / 32), 32}, s);
-  if (teams_fit(c, L)) return launch_ck45_teams(c->km_flags, a, L, s);
+  if (teams_fit(c, L)) {
+    // a plain launch in blocks of one team, whatever its own: five of those fit on an SM, but
+    // two of two teams and one of three or four, whose rest would wait for the first ones
+    // (24,320 x 2 in blocks of two and four teams 44.3 and 47.1 ms, of one 27.4; 20,000 x 2 in
+    // blocks of three 43.5, of one 26.3).  Persistent launches keep theirs: resident blocks claim
+    // for those that wait (20,000 x 2 in 128 x 2 25.6)
+    if (!a.persistent) L = AdaptLaunch{(c->n + 31) / 32, 32};
+    return launch_ck45_teams(c->km_flags, a, L, s);
+  }
   return launch_ck45(c->sys, c->km_flags, a, L, s);
 }
 
