@@ -17,7 +17,7 @@ namespace ens {
 cudaError_t launch_rk4(int sys, bool strict, const Rk4Args& a, int block, int spt, cudaStream_t s);
 cudaError_t launch_ck45(int sys, unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_fp32c(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
-cudaError_t launch_ck45_df(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
+cudaError_t launch_ck45_df(unsigned flags, bool unrolled, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_df_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_df_events(const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
 cudaError_t launch_ck45_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s);
@@ -266,12 +266,23 @@ bool valve_relay_fits(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L) {
          L.grid <= 4 * (int64_t)c->sm_count;
 }
 
-// The same for double-float phases, in teams of two or three (df64.cu): up to 6 per
-// SM, 8 in larger blocks (8 warps per SM, 131,044 x 2: 42.3 ms, plain 49.0)
+// The same for double-float phases, in teams of two or three (df64.cu): up to 6 per SM,
+// and 8 in persistent blocks of 7 or 8 (8 warps per SM, 131,044 x 2: 42.3 ms, plain 49.0)
 // (131,044 systems x 2 periods 41.9 ms against 45.4 in plain warps; 262,144 x 2
 // 83.7 against 62.1 in 12 plain warps per SM).
-bool df_teams_fit(const ens_ctx* c, AdaptLaunch L) {
-  return L.block <= 256 && L.grid * (L.block / 32) <= (L.block <= 192 ? 6 : 8) * (int64_t)c->sm_count;
+bool df_teams_fit(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L) {
+  return L.grid * (L.block / 32) <= (a.persistent && L.block > 192 ? 8 : 6) * (int64_t)c->sm_count;
+}
+
+// Whether the other double-float phases take the kernel with unrolled stages: where the
+// longest trials bound them, that is for up to 10 warps of systems per SM (37,000 x 2 in
+// blocks of 64: 25.4 ms, rolled 31.1; 45,000: 27.2 / 33.1; 65,536, 13 to 14 warps, random
+// order: 49.2 / 45.2) and, with one frequency, in up to 8 warps per SM that claim up to four
+// systems a lane (65,536 x 2 in 8 warps 30.5 / 33.9; 131,044, longest first, 30.8 / 33.4;
+// 262,144 57.1 / 51.1; two frequencies, 131,044: 83.3 / 74.3).
+bool df_unrolled(const ens_ctx* c, AdaptLaunch L) {
+  const int64_t lanes = L.grid * L.block, warp = 32 * (int64_t)c->sm_count;
+  return c->n <= 10 * warp || (!(c->km_flags & kKmDual) && lanes <= 8 * warp && c->n <= 4 * lanes);
 }
 
 // the adaptive kernel of the context's precision
@@ -279,9 +290,11 @@ cudaError_t launch_adaptive(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L,
   if (c->tol.prec == ENS_FP32_COMP) return launch_ck45_fp32c(c->km_flags, a, L, s);
   if (c->tol.prec == ENS_FP32X2) {
     if (c->sys == ENS_SYS_RELIEF_VALVE) return launch_ck45_df_events(a, L, s);
-    if (!df_teams_fit(c, L)) return launch_ck45_df(c->km_flags, a, L, s);
-    // a plain launch in blocks of two teams, whatever its own (16,384 x 2 in 8 warps a block 40.1 -> 26.7 ms)
-    if (!a.persistent && L.block > 64) L = AdaptLaunch{(c->n + 63) / 64, 64};
+    // a plain launch of up to 8 warps per SM in blocks of two, whatever its own, so that each SM
+    // gets its share (16,384 x 2 in 8 warps a block 40.1 -> 26.7 ms; above 6 warps, where as
+    // many teams fit, 37,000 x 2 in the one-warp kernel 25.4, in 8 teams a block 41.1)
+    if (!a.persistent && L.block > 64 && c->n <= 256 * (int64_t)c->sm_count) L = AdaptLaunch{(c->n + 63) / 64, 64};
+    if (!df_teams_fit(c, a, L)) return launch_ck45_df(c->km_flags, df_unrolled(c, L), a, L, s);
     return launch_ck45_df_teams(c->km_flags, a, L, s);
   }
   if (L.spt == 2) return launch_ck45_spt2(c->sys, c->km_flags, a, L, s);

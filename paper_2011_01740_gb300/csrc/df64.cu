@@ -90,7 +90,7 @@ __device__ __forceinline__ DF dmax(DF a, DF b) { return df::gt(a, b) ? a : b; }
 
 }  // namespace
 
-template <bool DUAL>
+template <bool DUAL, int UNROLL>
 __global__ void __launch_bounds__(256, 2) ck_phased_df_kernel(AdaptArgs a) {
   using namespace df;
   const double tau_end = a.t0 + a.phase_len;
@@ -181,10 +181,11 @@ __global__ void __launch_bounds__(256, 2) ck_phased_df_kernel(AdaptArgs a) {
         clamped = true;
       }
       const DF hd = from_double(h);
-      // The six stages as a rolled loop: the right-hand side and the forcing, 600
-      // instructions, appear once instead of six and five times (86 KB of code,
-      // whose fetch stalled: 262,144 systems x 2 periods 89.6 -> 60.8 ms with the
-      // packed sums).  Slopes are packed pairs (x, v); the first stage is
+      // The six stages as a rolled loop where many warps share an SM: the right-hand
+      // side and the forcing, 600 instructions, appear once instead of six and five
+      // times (86 KB of code, whose fetch stalled: 262,144 systems x 2 periods 89.6 ->
+      // 60.8 ms with the packed sums).  Few warps are bound by the longest trials, which
+      // the unrolled loop takes faster (launch_adaptive in abi.cu).  Slopes are packed pairs (x, v); the first stage is
       // evaluated after a rejection again, with the same inputs.
       nrhs += k1valid ? 5 : 6;
       k1valid = true;
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(256, 2) ck_phased_df_kernel(AdaptArgs a) {
       const DF2 yp = pack(y1, y2), h2 = both(hd);
       DF2 p1, p2, p3, p4, p5, p6;
       DF f5s, f5c;
-#pragma unroll 1
+#pragma unroll UNROLL
       for (int stage = 1; stage <= 6; ++stage) {
         DF x = y1, v = y2, fs = fks, fc = fkc;
         if (stage > 1) {
@@ -813,13 +814,18 @@ cudaError_t launch_ck45_df_teams(unsigned flags, const AdaptArgs& a, AdaptLaunch
   return cudaGetLastError();
 }
 
-cudaError_t launch_ck45_df(unsigned flags, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s) {
+cudaError_t launch_ck45_df(unsigned flags, bool unrolled, const AdaptArgs& a, AdaptLaunch L, cudaStream_t s) {
   if (a.n == 0) return cudaSuccess;
   if (a.n_phases <= 0) return cudaErrorInvalidValue;
   if (L.grid <= 0 || L.grid > 0x7fffffffLL || L.block <= 0) return cudaErrorInvalidConfiguration;
   const dim3 g((unsigned)L.grid), b((unsigned)L.block);
-  if (flags & kKmDual) ck_phased_df_kernel<true><<<g, b, 0, s>>>(a);
-  else ck_phased_df_kernel<false><<<g, b, 0, s>>>(a);
+  if (flags & kKmDual) {
+    if (unrolled) ck_phased_df_kernel<true, 6><<<g, b, 0, s>>>(a);
+    else ck_phased_df_kernel<true, 1><<<g, b, 0, s>>>(a);
+  } else {
+    if (unrolled) ck_phased_df_kernel<false, 6><<<g, b, 0, s>>>(a);
+    else ck_phased_df_kernel<false, 1><<<g, b, 0, s>>>(a);
+  }
   return cudaGetLastError();
 }
 

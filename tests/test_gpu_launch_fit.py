@@ -47,6 +47,7 @@ def _best_ms(ctx, launch, runs=3):
     (ens.ENS_FP64, False, 16000, _plain(32), [_plain(96)]),
     (ens.ENS_FP64, False, 20000, _plain(32), [_plain(64), _plain(96), _plain(128), _persistent(128, 2)]),
     (ens.ENS_FP64, True, 24320, _plain(32), [_plain(64), _plain(128), _persistent(128, 2)]),
+    (ens.ENS_FP32X2, False, 37000, _persistent(256, 1), [_plain(64), _plain(224), _plain(256), _persistent(224, 2)]),
 ])
 def test_no_shape_runs_in_two_waves(prec, dual, n, fits, launches):
     ctx = _context(n, prec, dual)
