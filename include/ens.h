@@ -300,8 +300,11 @@ int32_t ens_npar(const ens_ctx *ctx);
  *   with different tails can trade places as the horizon grows.  The claim
  *   order comes from the full solve's one-phase pilot, computed once.
  * The context's outputs hold the last candidate's shortened solve afterwards.
- * The choice and its table are cached per (system, solver, precision, n,
- * phases, transient phases, horizon, device) for the process. */
+ * The choice and its table are cached for the process, per (system, solver,
+ * precision, n, phases, transient phases, horizon, device, rtol, atol, and for
+ * Keller-Miksis whether any system has a second frequency or an exponent other
+ * than 21/5).  When ens_set_inputs changes the latter, the context goes back to
+ * its default launch (use_graph is kept). */
 ens_status ens_autotune(ens_ctx *ctx, void *stream, ens_launch *best);
 
 /* The candidates timed by the context's last ens_autotune, in the order

@@ -58,7 +58,8 @@ struct ens_ctx {
   unsigned* hist = nullptr;     // histogram scratch of the claim-order sort
   Scratch* scratch = nullptr;
   ens_launch launch{};
-  bool launch_set = false;   // by the caller or the tuner; else it follows the parameters
+  // who chose it: what the caller set stays, the default and the tuner's choice follow the parameters
+  enum { kDefault, kTuned, kCaller } launch_by = kDefault;
   // CUDA graph of one solve
   cudaGraphExec_t gexec = nullptr;
   cudaStream_t graph_stream = nullptr;
@@ -588,8 +589,10 @@ ens_status check_tol(ens_ctx* c, ens_solver solver, ens_system sys, const ens_to
 namespace {
 
 // tuned launch and its candidate table per (system, solver, precision, n,
-// phases, transient phases, horizon, device)
-std::map<std::tuple<int, int, int, int64_t, int, int, double, int>, std::pair<ens_launch, std::vector<ens_tune_row>>>
+// phases, transient phases, horizon, device, tolerances, kind of parameters: the
+// kernels and the candidates depend on km_flags)
+std::map<std::tuple<int, int, int, int64_t, int, int, double, int, double, double, unsigned>,
+         std::pair<ens_launch, std::vector<ens_tune_row>>>
     g_tune_cache;
 
 }  // namespace
@@ -712,7 +715,12 @@ ens_status ens_set_inputs(ens_ctx* c, const double* params, const double* y0, vo
     if (st != ENS_OK) return st;
     if (was != c->km_flags) {
       c->graph_valid = false;
-      if (!c->launch_set) c->launch = default_launch(c);
+      if (c->launch_by != ens_ctx::kCaller) {
+        const int graph = c->launch.use_graph;
+        c->launch = default_launch(c);
+        c->launch.use_graph = graph;
+        c->launch_by = ens_ctx::kDefault;
+      }
     }
   }
   return ENS_OK;
@@ -734,7 +742,7 @@ ens_status ens_set_launch(ens_ctx* c, const ens_launch* cfg) {
     return ENS_ENOTSUP;
   }
   c->launch = L;
-  c->launch_set = cfg != nullptr;
+  c->launch_by = cfg ? ens_ctx::kCaller : ens_ctx::kDefault;
   c->graph_valid = false;
   return ENS_OK;
 }
@@ -852,14 +860,15 @@ ens_status ens_autotune(ens_ctx* c, void* stream, ens_launch* best) {
   }
   const double horizon = c->solver == ENS_RK4 ? (double)c->tol.n_steps : c->t1 - c->t0;
   const auto key = std::make_tuple((int)c->sys, (int)c->solver, (int)c->tol.prec, c->n,
-                                   (int)c->tol.n_phases, (int)c->tol.n_transient, horizon, c->device);
+                                   (int)c->tol.n_phases, (int)c->tol.n_transient, horizon, c->device, c->tol.rtol,
+                                   c->tol.atol, c->km_flags);
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
     auto it = g_tune_cache.find(key);
     if (it != g_tune_cache.end()) {
       const bool graph = c->launch.use_graph;
       c->launch = it->second.first;
-      c->launch_set = true;
+      c->launch_by = ens_ctx::kTuned;
       c->launch.use_graph = graph;
       c->tune_rows = it->second.second;
       c->graph_valid = false;
@@ -999,7 +1008,7 @@ ens_status ens_autotune(ens_ctx* c, void* stream, ens_launch* best) {
   if (st != ENS_OK) return st;
   best_L.use_graph = c->launch.use_graph;
   c->launch = best_L;
-  c->launch_set = true;
+  c->launch_by = ens_ctx::kTuned;
   c->graph_valid = false;
   {
     std::lock_guard<std::mutex> lk(g_tune_mu);
