@@ -289,8 +289,9 @@ int32_t ens_npar(const ens_ctx *ctx);
  *   to 1e9 system-steps, else on 1/8 of the steps.
  *   Adaptive: persistent launches of 3 to 24 warps per SM with longest-first
  *   claiming (FP64 Keller-Miksis phases of more than 64 systems per SM also 1
- *   and 2), the best residency without it, a plain launch and, where the
- *   kernel exists, two systems per thread at 6 and 8 warps per SM, each on
+ *   and 2), the launch of an untuned context, the best of these without that
+ *   order, a plain launch (the untuned context's, if that is plain) and, where
+ *   the kernel exists, two systems per thread at 6 and 8 warps per SM, each on
  *   1/8 of the phases (or of the time span) of every system -- the horizon is
  *   cut, not the ensemble, so the balance between throughput and the
  *   longest system's chain stays that of the full solve; the fraction is

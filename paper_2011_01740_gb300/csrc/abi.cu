@@ -962,26 +962,25 @@ ens_status ens_autotune(ens_ctx* c, void* stream, ens_launch* best) {
       frac *= 0.5;
       ms *= 0.5f;
     }
-    // warps per SM -> (block, blocks per SM)
+    // warps per SM, block, blocks per SM
     const int shapes[][3] = {{3, 96, 1},  {4, 128, 1},  {5, 160, 1},  {6, 192, 1},  {7, 224, 1},
                              {8, 256, 1}, {12, 192, 2}, {16, 256, 2}, {24, 256, 3}};
-    // relays, where not every system starts at once
-    if (has_teams(c) && c->n > 64 * (int64_t)c->sm_count)
+    // the launch of an untuned context, where the lists below lack it
+    const ens_launch untuned = default_launch(c);
+    const bool plain = untuned.mode == ENS_LAUNCH_PLAIN;
+    bool listed = plain;
+    for (const auto& sh : shapes) listed |= sh[1] == untuned.block && sh[2] == untuned.blocks_per_sm;
+    const bool relays = has_teams(c) && c->n > 64 * (int64_t)c->sm_count;   // not every system starts at once
+    listed |= relays && untuned.block == 32;
+    if (st == ENS_OK && !listed) st = consider(mk(untuned.mode, untuned.block, untuned.blocks_per_sm, untuned.cost_order, 1));
+    if (relays)
       for (const int bps : {1, 2})
         if (st == ENS_OK) st = consider(mk(ENS_LAUNCH_PERSISTENT, 32, bps, 1, 1));
-    int best_w = 0;
-    for (const auto& sh : shapes) {
-      if (st != ENS_OK) break;
-      const float before = best_ms;
-      st = consider(mk(ENS_LAUNCH_PERSISTENT, sh[1], sh[2], 1, 1));
-      if (best_ms < before) best_w = sh[0];
-    }
-    // the same residency without longest-first claiming, and a plain launch
-    if (st == ENS_OK && best_w > 0) {
-      for (const auto& sh : shapes)
-        if (sh[0] == best_w) st = consider(mk(ENS_LAUNCH_PERSISTENT, sh[1], sh[2], 0, 1));
-    }
-    if (st == ENS_OK) st = consider(mk(ENS_LAUNCH_PLAIN, 128, 0, 0, 1));
+    for (const auto& sh : shapes)
+      if (st == ENS_OK) st = consider(mk(ENS_LAUNCH_PERSISTENT, sh[1], sh[2], 1, 1));
+    // the best of these without longest-first claiming, and a plain launch
+    if (st == ENS_OK) st = consider(mk(ENS_LAUNCH_PERSISTENT, best_L.block, best_L.blocks_per_sm, 0, 1));
+    if (st == ENS_OK) st = consider(mk(ENS_LAUNCH_PLAIN, plain ? untuned.block : 128, 0, 0, 1));
     // two systems per thread where the kernel exists: 6 and 8 warps per SM
     // (236 registers a thread leave room for 8), longest first
     for (const int b : {96, 128}) {

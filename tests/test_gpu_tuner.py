@@ -1,6 +1,7 @@
 """What the tuner's choice depends on: a choice made for one kind of parameters or
 tolerance is not taken over for another, and what it chose for one kind is dropped when
-the context gets parameters of the other."""
+the context gets parameters of the other.  The launch that an untuned context takes is
+among the candidates."""
 import numpy as np
 import pytest
 
@@ -92,3 +93,29 @@ def test_a_tuned_launch_goes_with_the_parameters_it_was_made_for(use_graph):
     finally:
         ens.ens_destroy(ctx)
         ens.ens_destroy(fresh)
+
+
+@pytest.mark.parametrize("case,prec,n", [("valve", ens.ENS_FP64, 500), ("valve", ens.ENS_FP32X2, 500),
+                                         ("km", ens.ENS_FP64, 500), ("km", ens.ENS_FP64, 1300 * SMS),
+                                         ("km", ens.ENS_FP64, 1700 * SMS), ("km", ens.ENS_FP64, 150 * SMS),
+                                         ("km", ens.ENS_FP32_COMP, 500), ("km", ens.ENS_FP32_COMP, 1300 * SMS),
+                                         ("km", ens.ENS_FP32X2, 200 * SMS), ("km", ens.ENS_FP32X2, 1300 * SMS)])
+def test_the_untuned_launch_is_a_candidate(case, prec, n):
+    if case == "valve":
+        w = W.prv(n, t1=2.0)
+        t = w["tol"]
+        ctx = ens.ens_create(ens.ENS_SYS_RELIEF_VALVE, n, w["params"], w["y0"], (0.0, 2.0), ens.ENS_RKCK45,
+                             ens.make_tol(rtol=1e-7, atol=1e-7, dt0=t.dt0, dt_max=t.dt_max, event_tol=t.event_tol,
+                                          prec=prec))
+    else:
+        C, y0, tol = _km(n, n_phases=1, rtol=1e-5, atol=1e-5, prec=prec)
+        ctx = _create(C, y0, tol)
+    try:
+        d = ens.ens_get_launch(ctx)
+        untuned = (d.mode, d.block, d.blocks_per_sm, d.cost_order, 1)
+        ens.ens_autotune(ctx)
+        rows = ens.ens_autotune_table(ctx)
+        first = [s for s, r in zip(_shapes(ctx), rows) if r["horizon_frac"] == rows[0]["horizon_frac"]]
+        assert untuned in first and len(set(first)) == len(first)      # none of them twice
+    finally:
+        ens.ens_destroy(ctx)
