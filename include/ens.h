@@ -389,7 +389,11 @@ ens_status ens_mlp_loss_grad(ens_mlp *m, int64_t n, const float *x, const float 
                              float *grad, void *stream);
 /* Train on n samples (x [n][2], y [n][2]) with shuffled mini-batches; loss_hist
  * (host, may be NULL) receives the mean per-sample loss of each epoch and
- * member ([epochs][members]).  Synchronous. */
+ * member ([epochs][members]).  Synchronous.  The network keeps the buffers of
+ * the largest run so far for the next one: 8 bytes a sample on the device and
+ * 12 of page-locked host memory, up to 2^24 samples (134 and 201 MB); those of
+ * a run over more samples are pageable and given back when it ends, as all are
+ * by ens_mlp_destroy. */
 ens_status ens_mlp_train(ens_mlp *m, int64_t n, const float *x, const float *y, const ens_train_cfg *cfg,
                          float *loss_hist, void *stream);
 /* Fused ensemble inference: mean[n], stdv[n] (population standard deviation

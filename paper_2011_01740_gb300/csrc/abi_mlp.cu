@@ -7,6 +7,7 @@
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
+#include <cstdlib>
 #include <cstring>
 #include <new>
 #include <vector>
@@ -38,11 +39,13 @@ struct ens_mlp {
   float* block = nullptr;         // tcgen05: FP32 dz and gelu(z_4), see TrainTcArgs
   __nv_bfloat16* tile = nullptr;  // tcgen05: operand tiles, see TrainTcArgs
   // shuffles of a training run over up to shuffle_cap samples: draws and permutation
-  // on the device; draws and two permutations in pinned memory
+  // on the device; on the host draws and two permutations in pinned memory, or draws and
+  // one permutation in pageable memory
   int64_t shuffle_cap = 0;
   int32_t* draw_d = nullptr;
   int32_t* perm_d = nullptr;
-  int32_t* shuffle_h = nullptr;   // [3][shuffle_cap]
+  int32_t* shuffle_h = nullptr;   // [pinned ? 3 : 2][shuffle_cap]
+  bool shuffle_pinned = false;
   cudaEvent_t drawn = nullptr;
   cudaEvent_t copied[2] = {nullptr, nullptr};
   float* hist = nullptr;          // [hist_cap] loss sums of epochs and members
@@ -121,13 +124,16 @@ void free_batch(ens_mlp* m) {
 
 __host__ __device__ constexpr df::DF pair_of(double x) { return df::DF{(float)x, (float)(x - (double)(float)x)}; }
 
-// the shuffle buffers of a run over more samples than this are given back after it
+// The shuffle buffers of a run over more samples than this are given back after it, and
+// those on the host are pageable: page-locked ones, 25 GB for the most samples, are no
+// faster where each run makes them (2^25 samples, one epoch: 295 ms, page-locked 289 to 489).
 constexpr int64_t kKeepShuffle = 1 << 24;
 
 void free_shuffle(ens_mlp* m) {
   cudaFree(m->draw_d);
   cudaFree(m->perm_d);
-  cudaFreeHost(m->shuffle_h);
+  if (m->shuffle_pinned) cudaFreeHost(m->shuffle_h);
+  else free(m->shuffle_h);
   m->draw_d = m->perm_d = m->shuffle_h = nullptr;
   m->shuffle_cap = 0;
 }
@@ -140,7 +146,14 @@ ens_status ensure_shuffle(ens_mlp* m, int64_t n, int64_t hist) {
     free_shuffle(m);
     e = cudaMalloc(&m->draw_d, n * sizeof(int32_t));
     if (e == cudaSuccess) e = cudaMalloc(&m->perm_d, n * sizeof(int32_t));
-    if (e == cudaSuccess) e = cudaMallocHost(&m->shuffle_h, 3 * n * sizeof(int32_t));
+    if (e == cudaSuccess) {
+      m->shuffle_pinned = n <= kKeepShuffle && cudaMallocHost(&m->shuffle_h, 3 * n * sizeof(int32_t)) == cudaSuccess;
+      if (!m->shuffle_pinned) {
+        cudaGetLastError();
+        m->shuffle_h = static_cast<int32_t*>(malloc(2 * n * sizeof(int32_t)));
+        if (!m->shuffle_h) e = cudaErrorMemoryAllocation;
+      }
+    }
     if (e == cudaSuccess) m->shuffle_cap = n;
     else free_shuffle(m);
   }
@@ -641,7 +654,8 @@ ens_status ens_mlp_train(ens_mlp* m, int64_t n, const float* x, const float* y, 
   int64_t step = 0;
   if (e == cudaSuccess && cfg->epochs > 0) draw_epoch(0);
   for (int ep = 0; ep < cfg->epochs && e == cudaSuccess; ++ep) {
-    int32_t* perm = m->shuffle_h + (1 + (ep & 1)) * m->shuffle_cap;
+    // a copy from pageable memory has read it when the call returns
+    int32_t* perm = m->shuffle_h + (m->shuffle_pinned ? 1 + (ep & 1) : 1) * m->shuffle_cap;
     if (ep >= 2) e = cudaEventSynchronize(m->copied[ep & 1]);
     for (int64_t i = 0; i < n; ++i) perm[i] = (int32_t)i;
     if (e == cudaSuccess) e = cudaEventSynchronize(m->drawn);
