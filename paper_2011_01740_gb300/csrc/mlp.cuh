@@ -77,12 +77,6 @@ __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(
 __device__ __forceinline__ float gelu_grad(float z) {
   return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) + z * 0.39894228040143268f * __expf(-0.5f * z * z);
 }
-// both from one erf evaluation (the same expressions as gelu and gelu_grad)
-__device__ __forceinline__ void gelu_and_grad(float z, float& h, float& g) {
-  const float phi2 = 1.0f + erff(z * 0.70710678118654752f);
-  h = 0.5f * z * phi2;
-  g = 0.5f * phi2 + z * 0.39894228040143268f * __expf(-0.5f * z * z);
-}
 
 // gelu of two values, and of two sums with a bias, the operations around erff in
 // packed FP32 pairs: the same bits as gelu (compared over all floats) in 27.5 issue
@@ -95,7 +89,8 @@ __device__ __forceinline__ void gelu2(df::F2 z, float& a, float& b) {
   const F2 phi2 = add_f(f2(erff(s), erff(t)), f2(1.0f, 1.0f));
   unpack(mul_f(mul_f(z, f2(0.5f, 0.5f)), phi2), &a, &b);
 }
-// gelu_and_grad of two values, with its multiply-adds as the compiler contracts them
+// gelu and gelu_grad of two values, each pair from one erf evaluation; the multiply-adds
+// are those that the compiler contracts the expressions above to
 __device__ __forceinline__ void gelu_and_grad2(df::F2 z, float& ha, float& hb, float& ga, float& gb) {
   using namespace df;
   float s, t, u, v;
