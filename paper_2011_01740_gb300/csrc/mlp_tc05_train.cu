@@ -338,7 +338,9 @@ namespace {
 // A group of 128 threads (thread = feature f) walks the 32-sample blocks
 // quarter(0), quarter(1), .. of one array over a slice's rows [lo, hi), in
 // order: use(d, row in the block, pairs of the block's rows).  Blocks arrive through a ring of
-// kDepth; pairs (may be null) are the slice's [rows][2] x or dout.
+// kDepth; pairs (may be null) are the slice's [rows][2] x or dout.  After a wait that
+// expired a thread waits no more, and the one that copies starts no copy on that
+// barrier again and ends with a wait for those under way.
 template <class Quarter, class Use>
 __device__ __forceinline__ bool walk_blocks(int grp, const float* src, const float* pairs, int64_t lo, int64_t hi,
                                             unsigned char* ring, unsigned char* pair_ring, uint32_t bars,
@@ -347,6 +349,7 @@ __device__ __forceinline__ bool walk_blocks(int grp, const float* src, const flo
   const int at = ((f & 31) >> 2) * (kBlock / 8) + (f >> 5) * 128 + (f & 3);
   const uint32_t ring_a = smem_u32(ring), pair_a = smem_u32(pair_ring);
   bool ok = true;
+  int64_t lost = 0;   // the block whose wait expired
   auto load = [&](int64_t k) {
     const int64_t g = quarter(k);
     if (f != 0 || 32 * g >= hi) return;
@@ -358,12 +361,16 @@ __device__ __forceinline__ bool walk_blocks(int grp, const float* src, const flo
               (uint32_t)kBlockBytes, bar);
     if (pairs) bulk_load(pair_a + slot * 256, pairs + 64 * g, pb, bar);
   };
+  auto arrived = [&](int64_t k) { return bar_wait(bars + 8 * (uint32_t)(k % kDepth), (uint32_t)((k / kDepth) & 1)); };
 #pragma unroll
   for (int k = 0; k < kDepth; ++k) load(k);
   for (int64_t k = 0; 32 * quarter(k) < hi; ++k) {
     const int64_t row = 32 * quarter(k);
     const uint32_t slot = (uint32_t)(k % kDepth);
-    ok &= bar_wait(bars + 8 * slot, (uint32_t)((k / kDepth) & 1));
+    if (ok && !arrived(k)) {
+      ok = false;
+      lost = k;
+    }
     const float* d = reinterpret_cast<const float*>(ring + slot * kBlockBytes) + at;
     const float2* q = reinterpret_cast<const float2*>(pair_ring + slot * 256);
     if (row >= lo && row + 32 <= hi) {
@@ -374,8 +381,10 @@ __device__ __forceinline__ bool walk_blocks(int grp, const float* src, const flo
         if (row + i >= lo && row + i < hi) use(d[4 * i], q + i);
     }
     asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory");   // the slot has been read
-    load(k + kDepth);
+    if (ok) load(k + kDepth);
   }
+  if (!ok && f == 0)
+    for (int64_t k = lost; k < lost + kDepth && 32 * quarter(k) < hi; ++k) arrived(k);
   return ok;
 }
 
@@ -460,19 +469,27 @@ __global__ void __launch_bounds__(kT, 1) mlp_wgrad_tc05_kernel(TrainTcArgs a) {
         bulk_load(slot, src + ((int64_t)c * 6 + (l - 2)) * H * H, kM, bar);
         bulk_load(slot + kM, src + ((int64_t)c * 6 + (7 - l)) * H * H, kM, bar);
       };
+      auto arrived = [&](int c) { return bar_wait(full + (c & 1) * 8, (uint32_t)(c >> 1) & 1); };
       load(0);
       if (chunks > 1) load(1);
-      for (int c = 0; c < chunks; ++c) {
-        const uint32_t slot = base + (uint32_t)(c & 1) * 2 * kM, par = (uint32_t)(c >> 1) & 1;
-        ok &= bar_wait(full + (c & 1) * 8, par);
-        mma_128<true, true>(tmem, slot + kM, slot, c > 0);
-        mma_commit(c + 1 < chunks ? freed + (c & 1) * 8 : smem_u32(bars + 4));
-        if (c + 2 < chunks) {
-          ok &= bar_wait(freed + (c & 1) * 8, par);
-          load(c + 2);
+      for (int c = 0; c < chunks && ok; ++c) {
+        const uint32_t slot = base + (uint32_t)(c & 1) * 2 * kM;
+        ok = arrived(c);
+        if (ok) {
+          mma_128<true, true>(tmem, slot + kM, slot, c > 0);
+          mma_commit(c + 1 < chunks ? freed + (c & 1) * 8 : smem_u32(bars + 4));
+          if (c + 2 < chunks) {
+            ok = bar_wait(freed + (c & 1) * 8, (uint32_t)(c >> 1) & 1);
+            if (ok) load(c + 2);
+          }
+        }
+        if (!ok) {   // the others wait for the products issued so far, this thread for the copies under way
+          mma_commit(smem_u32(bars + 4));
+          arrived(c);
+          if (c + 1 < chunks) arrived(c + 1);
+          atomicOr(a.error, 1u);
         }
       }
-      if (!ok) atomicOr(a.error, 1u);
     }
   } else if (grp < 2) {
     // bias gradient: group 0 takes the first 64 samples of every tile, group 1
