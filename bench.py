@@ -30,34 +30,35 @@ sys.path.insert(0, ROOT)
 
 from paper_2011_01740_gb300 import workloads as W  # noqa: E402
 
-# FP64 flops (DFMA = 2, DADD = DMUL = 1) executed per Cash-Karp trial step of
-# the Keller-Miksis kernel, and per RK4 step of the x' = x^2 - p and Lorenz
-# kernels, from the ncu instruction counters of profiles/ (None until
-# measured: the roofline then reports achieved = null).
-FLOPS_PER_KM_TRIAL = 340.19  # 135.68 DFMA + 65.86 DMUL + 2.98 DADD per trial (profiles/)
-# all FP64 thread instructions per trial, for the FP64 pipe's issue fraction
-FP64_INST_PER_KM_TRIAL = 204.52
+# Arithmetic of one work unit: a multiply-add counts 2 flops, a product or a sum 1,
+# as the kernels issued it (ncu instruction counters, profiles/) before products and
+# sums went out as multiply-adds by 1 or -0 and in packed pairs; both do the same
+# operations.  None until measured: the fractions are then null.
+FLOPS_PER_KM_TRIAL = 340.19  # Keller-Miksis Cash-Karp trial: 135.68 FMA + 65.86 products + 2.98 sums
+# FP64 pipe slots (lanes) per trial of the benchmarked launch, counted on the team
+# kernel: its first stage is evaluated ahead, for rejected trials too, and lanes that
+# ran out of systems go on with their warp.  The one-warp kernel issues 204.52.
+FP64_INST_PER_KM_TRIAL = 208.27
 # The same trial in its all-FP64 form (the forcing's sine and cosine, the
 # fifth root, the polytropic power and the error norm's reciprocals as FP64
 # arithmetic: 232.61 DFMA + 121.70 DMUL + 2.98 DADD, profiles/); the
 # fixed-point evaluations on the integer pipe take 250 of these flops off the
-# FP64 pipe.  Reported beside the executed count as the trial's FP64-form work.
+# FP64 pipe.  Reported beside the trial's own flops as its FP64-form work.
 FLOPS_FP64_FORM_KM_TRIAL = 589.91
 # DRAM bytes (read + write) of one benchmarked Keller-Miksis launch, from the
-# one-pass ncu capture in profiles/ (inputs 15.7 MB read once, 134 MB of
-# per-period accessories written once); None once the kernel changes.
+# one-pass ncu capture in profiles/ (inputs 15.7 MB, read once where they do not
+# stay in L2, 134 MB of per-period accessories, part of which L2 still holds at the
+# end); None once the kernel changes.
 KM_LAUNCH_DRAM_BYTES = 28436992 + 110093568
 FLOPS_PER_X2P_STEP = 21.0     # 10 DFMA + 1 DADD (Sec. 3.2.2 counters; kernel counted by ncu)
-FLOPS_PER_LORENZ_STEP = 75.0  # 30 DFMA + 8 DMUL + 7 DADD per step of the fast kernel
-# executed flops per trial of the other adaptive kernels (ncu counts,
-# profiles/; None until measured: their fractions are then null)
-FLOPS_PER_VALVE_TRIAL = 219.10        # FP64: 84.83 DFMA + 35.34 DMUL + 14.10 DADD, ck_events_kernel
+FLOPS_PER_LORENZ_STEP = 75.0  # 31 DFMA + 7 DMUL + 6 DADD per step of the fast kernel
+FLOPS_PER_VALVE_TRIAL = 219.10        # FP64: 84.83 FMA + 35.34 products + 14.10 sums
 # the valve trial in its all-FP64 form (square root, fifth root and reciprocals
 # as FP64 arithmetic: 115.0 DFMA + 57.5 DMUL + 14.1 DADD, profiles/)
 FLOPS_FP64_FORM_VALVE_TRIAL = 301.59
-FLOPS_FP32_PER_FP32C_TRIAL = 1516.0   # FP32: 441.1 FFMA + 162.4 FMUL + 471.4 FADD, ck_phased_fp32c_kernel
-FLOPS_FP32_PER_DF_TRIAL = 5277.6      # FP32: 746.1 FFMA + 454.9 FMUL + 3330.5 FADD, ck_phased_df_kernel
-FLOPS_FP32_PER_DF_VALVE_TRIAL = 3173.5  # FP32, ck_events_df_kernel
+FLOPS_FP32_PER_FP32C_TRIAL = 1516.0   # FP32: 441.1 FMA + 162.4 products + 471.4 sums, split precision
+FLOPS_FP32_PER_DF_TRIAL = 5277.6      # FP32: 746.1 FMA + 454.9 products + 3330.5 sums, double-float
+FLOPS_FP32_PER_DF_VALVE_TRIAL = 3173.5  # FP32, double-float valve
 # FP32 peak: 152 SMs x 128 FP32 lanes x 2 flop x 2.07 GHz
 FP32_PEAK = 152 * 128 * 2.0 * 2070.0e6
 
@@ -255,7 +256,7 @@ def run_ours(args):
         kernel_ms, kernel_src = float(np.mean(kernel_ms_steps)), "main-kernel CUDA events (ens_kernel_ms)"
     else:
         kernel_ms, kernel_src = total_ms / args.steps, "whole solve (pilot and ordering included)"
-    roofline = km_roofline(trials_local, kernel_ms, steps_local / args.steps)
+    roofline = km_roofline(trials_local, kernel_ms, steps_local / args.steps, launch)
     roofline["duration_source"] = kernel_src
 
     secondary = {}
@@ -332,21 +333,23 @@ def run_ours(args):
         dist.destroy_process_group()
 
 
-def km_roofline(trials: float, kernel_ms: float, accepted: float) -> dict:
-    """Roofline of the FP64 Keller-Miksis phase kernel: executed FP64 flops
-    per trial (ncu counts, profiles/) x trials / main-kernel time against the
-    FP64 peak derived from the clocks; with the FP64 instruction issue
-    fraction and the accepted share of the trials."""
+def km_roofline(trials: float, kernel_ms: float, accepted: float, launch) -> dict:
+    """Roofline of the FP64 Keller-Miksis phase kernel: the trials' FP64 flops
+    over the main kernel's time against the FP64 peak derived from the
+    clocks; with the FP64 instruction issue fraction (counted for the team
+    kernel) and the accepted share of the trials."""
     achieved = FLOPS_PER_KM_TRIAL * trials / (kernel_ms / 1e3) / 1e12 if FLOPS_PER_KM_TRIAL else None
+    teams = launch.block <= 160 and launch.block // 32 * launch.blocks_per_sm <= 5
+    kernel = "ck_phased_teams_kernel" if teams else "ck_phased_kernel"
     return {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK / 1e12, "unit": "TFLOP/s",
             "frac": (achieved / (FP64_PEAK / 1e12)) if achieved else None,
-            "traffic": KM_LAUNCH_DRAM_BYTES, "kernel": "ck_phased_teams_kernel<KellerMiksis<false, true>, 0>",
+            "traffic": KM_LAUNCH_DRAM_BYTES, "kernel": kernel + "<KellerMiksis<false, true>, 0>",
             "peak_source": "derived: 152 SMs x 4 FP64 flop/clk/SM x 2070 MHz (nominal 1.25 TFLOP/s)",
             "flops_per_trial": FLOPS_PER_KM_TRIAL, "trials_per_launch": trials,
             "kernel_ms": kernel_ms,
-            "fp64_inst_per_trial": FP64_INST_PER_KM_TRIAL,
+            "fp64_inst_per_trial": FP64_INST_PER_KM_TRIAL if teams else None,
             "fp64_issue_frac": (FP64_INST_PER_KM_TRIAL * trials / (kernel_ms / 1e3) / FP64_INST_PEAK
-                                if FP64_INST_PER_KM_TRIAL else None),
+                                if teams and FP64_INST_PER_KM_TRIAL else None),
             # the trial's flops in its all-FP64 form over the same time: what an
             # FP64-only kernel would have to reach to match this one
             "fp64_form_frac": FLOPS_FP64_FORM_KM_TRIAL * trials / (kernel_ms / 1e3) / FP64_PEAK,
@@ -1046,18 +1049,21 @@ def run_profile_case(case: str):
         ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS, C.shape[1], C, km["y0"], (0.0, 1.0),
                              ens.ENS_RKCK45, tol)
         ens.ens_set_launch(ctx, ens.make_launch(block=160, blocks_per_sm=1, cost_order=1))
-    elif case == "km_full2":
-        # all 131,044 systems, 2 periods: the instruction mix of the benchmarked kernel
+    elif case in ("km_full2", "km_full2_12w", "km_df_full2"):
+        # all 131,044 systems, 2 periods: the instruction mix of the benchmarked kernel (teams), of the
+        # one-warp kernel that larger grids take (12 warps per SM), and of the double-float one
         km = km_slice(1, 0, n_phases=2)
         ph = km["phys"]
         C = ens.ens_km_coefficients(ph["pA1"], ph["f1"], ph["pA2"], ph["f2"], ph["theta"], ph["RE"],
                                     km["liquid"])
         t = km["tol"]
         tol = ens.make_tol(rtol=t.rtol, atol=t.atol, dt0=t.dt0, dt_min=t.dt_min, dt_max=t.dt_max,
-                           n_phases=t.n_phases, phase_len=t.phase_len)
+                           n_phases=t.n_phases, phase_len=t.phase_len,
+                           prec=ens.ENS_FP32X2 if case == "km_df_full2" else ens.ENS_FP64)
         ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS, C.shape[1], C, km["y0"], (0.0, 1.0),
                              ens.ENS_RKCK45, tol)
-        ens.ens_set_launch(ctx, ens.make_launch(block=160, blocks_per_sm=1, cost_order=0))
+        shape = (160, 1) if case == "km_full2" else (128, 3)
+        ens.ens_set_launch(ctx, ens.make_launch(block=shape[0], blocks_per_sm=shape[1], cost_order=0))
     elif case == "km_fp32c":
         km = km_slice(1, 0, n_phases=2)
         idx = W.subsample(km["phys"]["pA1"].size, 16384)
@@ -1122,6 +1128,8 @@ def run_profile_case(case: str):
                            prec=ens.ENS_FP32X2 if case == "prv_df" else ens.ENS_FP64)
         ctx = ens.ens_create(ens.ENS_SYS_RELIEF_VALVE, 8192, wl["params"], wl["y0"], (t.t0, t.t1),
                              ens.ENS_RKCK45, tol)
+        if case == "prv":   # the one-warp kernel of large ensembles; blocks of 32 would run in relays
+            ens.ens_set_launch(ctx, ens.make_launch(mode=ens.ENS_LAUNCH_PLAIN, block=64, blocks_per_sm=0))
     elif case in ("x2p", "lorenz"):
         wl = W.x2p(1 << 20) if case == "x2p" else W.lorenz(16384)
         sysid = ens.ENS_SYS_TOY_X2P if case == "x2p" else ens.ENS_SYS_LORENZ
