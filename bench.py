@@ -284,7 +284,7 @@ def run_ours(args):
         secondary["km_work_precision_16384f"] = run_work_precision(ens, torch, stream, dev)
         secondary["km_frequency_response_46080f"] = run_frequency_response(ens, torch, stream, dev)
         secondary["km_dual_frequency_362x362"] = run_dual_frequency(ens, torch, stream, dev, launch)
-        secondary["km_lyapunov_362x362"] = run_lyapunov(ens, torch, stream, dev, C_d, km, launch)
+        secondary["km_lyapunov_362x362"] = run_lyapunov(ens, torch, stream, dev, C_d, km)
         secondary["km_dopri5_362x362"] = run_dopri5(ens, torch, stream, dev, ctx, C_d, y0_d, km, tol, launch,
                                                     total_ms / args.steps)
         secondary["km_fp32x2_362x362"] = run_fp32x2(ens, torch, stream, dev, ctx, C_d, y0_d, km, tol,
@@ -590,11 +590,12 @@ def run_screen(ens, torch, stream, dev, ctx, km, solve_ms, solve_steps, args):
     return r
 
 
-def run_lyapunov(ens, torch, stream, dev, C_d, km, launch, n_phases=64, n_transient=32):
+def run_lyapunov(ens, torch, stream, dev, C_d, km, n_phases=64, n_transient=32):
     """Largest Lyapunov exponent over the headline sweep: the Keller-Miksis
     tangent system, renormalised at every phase end on the device (Sec. 1,
     trajectory manipulation between phases), exponent = mean of the recorded
-    per-phase log growths (phases 33-64) per unit tau."""
+    per-phase log growths (phases 33-64) per unit tau.  The context's default
+    launch: one-warp trials want six warps per SM here, the headline's teams five."""
     n = km["phys"]["pA1"].size
     y0 = np.vstack([np.ones(n), np.zeros(n), np.ones(n), np.ones(n)])
     t = km["tol"]
@@ -603,7 +604,6 @@ def run_lyapunov(ens, torch, stream, dev, C_d, km, launch, n_phases=64, n_transi
     ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS_TANGENT, n, C_d, torch.from_numpy(y0).to(dev), (0.0, 1.0),
                          ens.ENS_RKCK45, tol)
     try:
-        ens.ens_set_launch(ctx, launch)
         ens.ens_solve(ctx, stream)
         ens.ens_sync(ctx)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -709,8 +709,8 @@ def run_dopri5(ens, torch, stream, dev, ck_ctx, C_d, y0_d, km, tol, launch, ck_m
 
 
 def _timed_km_solve(ens, torch, stream, dev, w, launch, n_transient=0, warm=False):
-    """One Keller-Miksis phase-mode solve of workload w on the given launch:
-    device time, counts and the recorded per-phase maxima."""
+    """One Keller-Miksis phase-mode solve of workload w on the given launch (None:
+    the context's default): device time, counts and the recorded per-phase maxima."""
     ph = w["phys"]
     n = ph["pA1"].size
     phys_d = [torch.from_numpy(ph[k]).to(dev) for k in ("pA1", "f1", "pA2", "f2", "theta", "RE")]
@@ -722,7 +722,9 @@ def _timed_km_solve(ens, torch, stream, dev, w, launch, n_transient=0, warm=Fals
     ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS, n, C, torch.from_numpy(w["y0"]).to(dev), (0.0, 1.0),
                          ens.ENS_RKCK45, tol)
     try:
-        ens.ens_set_launch(ctx, launch)
+        if launch is not None:
+            ens.ens_set_launch(ctx, launch)
+        shape = ens.ens_get_launch(ctx).as_dict()
         if warm:
             ens.ens_solve(ctx, stream)
             ens.ens_sync(ctx)
@@ -740,24 +742,18 @@ def _timed_km_solve(ens, torch, stream, dev, w, launch, n_transient=0, warm=Fals
         ens.ens_destroy(ctx)
     return {"ms": ms, "kernel_ms": kms, "status": st, "systems": n, "accepted_steps": float(nacc.sum()),
             "trials": float(nacc.sum() + nrej.sum()), "value": float(nacc.sum()) / (ms / 1e3),
-            "unit": "system-steps/s"}, acc
+            "unit": "system-steps/s", "launch": shape}, acc
 
 
 def run_frequency_response(ens, torch, stream, dev):
     """The paper's Keller-Miksis workload (Sec. 4.2): 46,080 frequencies at
     P_A1 = 1.5 bar, 1024 transient phases integrated and discarded, the
-    maxima of the next 64 recorded; one solve, a persistent launch with
-    longest-first claiming at 3 warps/SM."""
+    maxima of the next 64 recorded; one solve on the default launch."""
     w = W.km_frequency_response()
-    # 46,080 systems of 787k trials on average: the longest ones bound the run,
-    # and each warp's trials run fastest with few warps sharing the FP64 pipes
-    # (measured: 3 warps/SM 35.8 s, 4: 39.1 s, 5: 49.0 s, 8: 74.3 s, 10: 92.5 s)
-    res, acc = _timed_km_solve(ens, torch, stream, dev, w,
-                               ens.make_launch(block=96, blocks_per_sm=1, cost_order=1), n_transient=w["n_transient"])
+    res, acc = _timed_km_solve(ens, torch, stream, dev, w, None, n_transient=w["n_transient"])
     y1max = acc[0::2].max(axis=0)
     res["phases"] = {"transient": w["n_transient"], "recorded": w["tol"].n_phases - w["n_transient"]}
     res["y1max_range"] = [float(y1max.min()), float(y1max.max())]
-    res["launch"] = {"block": 96, "blocks_per_sm": 1, "cost_order": 1}
     return res
 
 
@@ -781,8 +777,7 @@ def run_fp32x2(ens, torch, stream, dev, ck_ctx, C_d, y0_d, km, tol, ck_ms):
                         n_phases=t.n_phases, phase_len=t.phase_len, prec=ens.ENS_FP32X2, timeout_s=900.0)
     ctx = ens.ens_create(ens.ENS_SYS_KELLER_MIKSIS, n, C_d, y0_d, (0.0, 1.0), ens.ENS_RKCK45, tol2)
     try:
-        # 7 warps/SM measured best (6: 1.80 s, 7: 1.79 s, 8: 1.97 s, 12: 2.71 s)
-        ens.ens_set_launch(ctx, ens.make_launch(block=224, blocks_per_sm=1, cost_order=1))
+        shape = ens.ens_get_launch(ctx).as_dict()   # the default: six teams per SM (5: 1.53 s, 6: 1.44, 8: 1.63)
         ens.ens_solve(ctx, stream)
         ens.ens_sync(ctx)
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -802,7 +797,7 @@ def run_fp32x2(ens, torch, stream, dev, ck_ctx, C_d, y0_d, km, tol, ck_ms):
     return {"ms": ms, "kernel_ms": kms, "status": st, "accepted_steps": float(nacc.sum()),
             "trials": float(nacc.sum() + nrej.sum()), "value": float(nacc.sum()) / (ms / 1e3),
             "unit": "system-steps/s", "speedup_vs_fp64": ck_ms / ms,
-            "launch": {"block": 224, "blocks_per_sm": 1, "cost_order": 1},
+            "launch": shape,
             "per_period_max_rel_diff_vs_fp64": {"median": float(np.median(rel)),
                                                 "p90": float(np.percentile(rel, 90)),
                                                 "frac_below_1e-8": float(np.mean(rel < 1e-8))}}
