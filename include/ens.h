@@ -165,7 +165,11 @@ typedef struct {
  *                  claims its next system from a device counter (atomicAdd)
  *                  when its current one finishes (work stealing), so uneven
  *                  adaptive step counts do not idle warps.
- *   block          threads per block (multiple of 32, 32..256).
+ *   block          lanes that hold systems, per block (multiple of 32, 32..256).
+ *                  Where the kernels spread a trial over several warps, a block
+ *                  has more threads than that; plain Keller-Miksis launches then
+ *                  go out in the blocks that fill the GPU evenly, whatever this
+ *                  says.  Results never depend on it.
  *   blocks_per_sm  persistent mode: resident blocks per SM (grid = SMs x this).
  *   use_graph      capture the launch sequence of ens_solve in a CUDA graph on
  *                  the first call and replay it afterwards.

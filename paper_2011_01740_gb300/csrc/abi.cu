@@ -110,16 +110,18 @@ ens_status cuda_fail(ens_ctx* c, cudaError_t e, const char* what) {
 //   with an order 22.7); above, one relay per SM that claims the longest first
 //   (19,200: 22.8, all at once in teams 35.0), then two (25,600: 25.1, one 27.6;
 //   51,200: 31.5, 3 teams 38.1), then 3 teams (65,536: 38.7, two relays 39.7), 4
-//   (90,000, kernel alone: 40.7, 3 teams 49.6), 5 (131,044 x 2: 52.4, 4 teams 59.0;
-//   x 4: 110.6, 6 plain warps 126.3), then 8 plain
+//   (90,000, kernel alone: 40.7, 3 teams 49.6), 5 (kernels alone, 560 systems per SM 41.9, 4
+//   teams 39.8; 640: 43.1 / 44.8; 131,044 x 2: 52.4 / 59.0; x 4: 110.6, 6 plain warps
+//   126.3), then 8 plain
 //   warps (200,000 x 2: 78.5, 5 teams 80.3), then 12 (262,144 x 2: 97.0, 5 teams
 //   105.1; 524,288: 199 / 209); other FP64 phases 5 warps (65,536: 57.6, 6 warps
 //   58.9), then 6 (131,044: 207 / 221 at 5), then 12.  Split precision, kernels
 //   alone: 4 (65,536 x 4: 14.2, 8 warps 16.0), then 8 (131,044: 16.2, 4 warps 20.5), 12
 //   (262,144: 19.5 / 23.1 at 8), 16 (524,288: 37.9 / 74.9 at 5), 24 from there.
 //   Double-float phases, kernels alone: teams on 2 of the sub-partitions (32,768 x 4:
-//   54.0, 3 teams 61.0), 3 (65,536: 61.9, 2 teams 80.6), 4 (90,000: 65.8, 3 teams 84.1),
-//   6 (131,044: 81.8, 4 teams 95.2), then 12 plain warps (262,144 x 2: 60.8, 8 warps
+//   54.0, 3 teams 61.0), 3 (65,536: 61.9, 2 teams 80.6), 4 (431 systems per SM x 4 64.7, 3
+//   teams 64.4; 439: 64.9 / 65.5; 90,000: 65.8 / 84.1), 6 (650 per SM x 2 38.0, 4 teams 36.0;
+//   710: 38.5 / 39.4; 131,044: 81.8 / 95.2), then 12 plain warps (262,144 x 2: 60.8, 8 warps
 //   71.1), then 16 (524,288 x 2: 111.6, 12 120.9).  Two frequencies leave the plain
 //   launch earlier, as four teams of three warps do not fit (19,200 x 2: 40.8 / 29.2).
 //   Valves take about the same number of steps each, and neighbours take them
@@ -268,9 +270,9 @@ bool valve_relay_fits(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L) {
 }
 
 // The same for double-float phases, in teams of two or three (df64.cu): up to 6 per SM,
-// and 8 in persistent blocks of 7 or 8 (8 warps per SM, 131,044 x 2: 42.3 ms, plain 49.0)
-// (131,044 systems x 2 periods 41.9 ms against 45.4 in plain warps; 262,144 x 2
-// 83.7 against 62.1 in 12 plain warps per SM).
+// and 8 in persistent blocks of 7 or 8 (131,044 x 2, longest first: 6 teams 40.5 ms, 8 44.5;
+// the one-warp kernel in 8 warps 44.9, in 12 60.2; 262,144 x 2: 6 teams 80.1, 12 warps
+// 63.6).
 bool df_teams_fit(const ens_ctx* c, const AdaptArgs& a, AdaptLaunch L) {
   return L.grid * (L.block / 32) <= (a.persistent && L.block > 192 ? 8 : 6) * (int64_t)c->sm_count;
 }

@@ -4,7 +4,7 @@
 // the fifth-order update, the error estimate and the step controller are
 // double-float pairs on the FP32 pipes (df.cuh, about 48 significant bits).
 // The FP64 pipe keeps the phase-local time tau, the step h and the forcing
-// sin / cos (sincos2pi_poly of rhs.cuh, split into pairs): 105 FP64 instructions
+// sin / cos (sincos2pi_poly of rhs.cuh, split into pairs): 107 FP64 instructions
 // per trial against 204.5 for the FP64 kernel.
 //
 // The algorithm is that of ck_phased_kernel with KellerMiksis (rhs.cuh,
@@ -288,8 +288,8 @@ __global__ void __launch_bounds__(256, 2) ck_phased_df_kernel(AdaptArgs a) {
 // starts, so a drive warp evaluates the forcing of the stages while the main
 // warp works on the stages before (messages as in rkck45_teams.cu).  Every
 // operation is that of ck_phased_df_kernel, so are the bits.
-// 65,536 systems x 4 periods 72.3 ms against 83.9 in the best plain shape, 1,073
-// x 2 32.2 against 38.1.
+// 65,536 systems x 4 periods 64.4 ms against 83.9 in the best one-warp shape, 1,073
+// x 2 25.4 against 38.1.
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -663,7 +663,7 @@ __global__ void __launch_bounds__(256) ck_events_df_kernel(AdaptArgs a) {
       }
       const DF hd = from_double(h);
       DF k2[D], k3[D], k4[D], k5[D], k6[D], x[D];
-      // Components 0 and 1 in packed pairs, component 2 alone: 3,200 -> 2,500
+      // Components 0 and 1 in packed pairs, component 2 alone: 3,200 -> 2,720
       // instructions a trial, 131,072 valves x 16 time units 39.6 -> 37.7 ms; the
       // FP32 pipe, which a packed instruction holds for two slots, is the bound now.
       const DF2 h2 = both(hd), yp = pack(y[0], y[1]);

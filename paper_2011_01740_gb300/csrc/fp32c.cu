@@ -271,9 +271,8 @@ __global__ void __launch_bounds__(256) ck_phased_fp32c_kernel(AdaptArgs a) {
       const float xb = (y0v.hi - 1.0f) + y0v.lo;
       const float vb = y1v.hi + y1v.lo;
       const float t2 = 2.0f * rn_f32(tau), h2 = 2.0f * hh;  // 2 RN(tau) = RN(2 tau)
-      // The sums in packed pairs take half the instructions, 1,960 -> 1,690 a trial
-      // (262,144 systems x 4 periods 19.4 -> 18.2 ms, 40,000, bound by the longest, 14.2 ->
-      // 12.0).  The stages stay unrolled, which lets them overlap (a rolled loop:
+      // The sums in packed pairs take half the instructions (262,144 systems x 4 periods
+      // 19.4 -> 18.2 ms, 40,000, bound by the longest, 14.2 -> 12.0).  The stages stay unrolled, which lets them overlap (a rolled loop:
       // 22.5 and 15.6); the first one is evaluated after a rejection again, with the
       // same inputs, for less than keeping it costs (18.3).
       nrhs += k1valid ? 5 : 6;

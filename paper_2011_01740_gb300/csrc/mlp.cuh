@@ -80,8 +80,9 @@ __device__ __forceinline__ float gelu_grad(float z) {
 
 // gelu of two values, and of two sums with a bias, the operations around erff in
 // packed FP32 pairs: the same bits as gelu (compared over all floats) in 27.5 issue
-// slots instead of 30 (screening 2048 x 2048 points with 4 members 8.30 -> 7.67 ms, a
-// training run of 130,682 samples x 2 epochs 3.25 -> 3.18)
+// slots instead of 30 (the whole screening kernel executes 27.7 instructions a GELU):
+// screening 2048 x 2048 points with 4 members 8.30 -> 7.67 ms, a training run of 130,682
+// samples x 2 epochs 3.25 -> 3.18
 __device__ __forceinline__ void gelu2(df::F2 z, float& a, float& b) {
   using namespace df;
   float s, t;

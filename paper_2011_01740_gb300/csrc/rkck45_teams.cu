@@ -25,7 +25,7 @@
 // 68.2 / 48.9, two frequencies and Dormand-Prince (6,097 x 2) 69.4 / 48.5; with
 // longest-first claiming 65,536 x 2 47.6 / 36.7, 131,044 x 6 189.4 (6 warps per
 // SM) / 166.4 (5 teams).  Registers allow 5 teams per SM, which keep the FP64 pipe
-// about 80 % busy; enough systems let more plain warps do better (262,144 x 2:
+// 82 % busy (131,044 x 64); enough systems let more plain warps do better (262,144 x 2:
 // 105.1 here, 97.0 with 12 plain warps), see teams_fit in abi.cu; up to two warps of
 // systems per SM the relay (rkck45_relay.cu) does.
 // What was tried: one helper warp for both kinds (37.4 ms on 1,073 systems; its
